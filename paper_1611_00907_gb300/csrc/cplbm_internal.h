@@ -40,14 +40,24 @@ struct EosParams {
 template <class T> struct EosT {
     int kind;
     T a, b, RT, aalpha, quarter_b, pr_c, pr_s2m1, pr_s2p1, rks_c;
+    T m2a;             // -2 a
 };
 
 // Physical constants of one lattice in the arithmetic type T, filled on the
 // host by set_consts: kernels do no double arithmetic and no double-to-float
 // conversion (GB300's FP64 pipe is narrow enough that two double divisions
 // per thread showed up as a busy FP64 pipe in the FP32 step).
+// The rest are the products a node's FP64 update multiplies by, so that its
+// kernels spend no instruction on them: the stencils are summed without
+// their factors 1/12 and 1/6 and the equilibria without omega w_i
+// (force_momentum, relax in device_common.cuh).
 template <class T> struct Consts {
     T tau, omega, kappa, rho_ref, mu_bottom, mu_top;   // omega = 1 / tau
+    T om1;                 // 1 - omega
+    T o9, o3, o12, o4;     // omega / 9, / 3, / 12, / 4
+    T no6;                 // -omega / 6
+    T t36, nt12;           // tau / 36, -tau / 12
+    T nk6;                 // -kappa / 6
     EosT<T> eos;
 };
 

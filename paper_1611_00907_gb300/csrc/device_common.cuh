@@ -102,32 +102,50 @@ __device__ __forceinline__ bool in_buffer(const Lattice &L, const void *base, lo
 // Bulk chemical potential psi'(rho): Eq. 18 (vdW), Eq. 21 (RK/RKS), Eq. 24
 // (PR), Eq. 27 (CS) without the -kappa lap(rho) term.
 // ---------------------------------------------------------------------------
-// FP64 reciprocal: the hardware's approximate reciprocal (PTX
-// rcp.approx.ftz.f64) refined by two Newton-Raphson steps r <- r + r (1 -
-// x r), each of which doubles the number of correct bits.  Within one ulp of
-// 1/x for normal x with a normal reciprocal (measured: the correctly
-// rounded value on 800 000 log-uniform samples), not guaranteed correctly
-// rounded as IEEE division is, at a fraction of its FP64-pipe instructions
-// (the GB300 FP64 pipe bounds the FP64 step).  Zero, infinite and NaN x give
-// NaN.
+// FP64 reciprocal: the hardware's approximate reciprocal r (PTX
+// rcp.approx.ftz.f64, which works on the upper 20 significand bits), then
+// one cubic step r (1 + e + e^2) with the residual e = 1 - x r: what is left
+// of the error is e^3, below 2^-56, a sixteenth of an ulp.  Three FP64-pipe
+// instructions, one less than the two Newton-Raphson steps that reach the
+// same (the GB300 FP64 pipe bounds the FP64 step).  Within one ulp of 1/x
+// for normal x with a normal reciprocal, not guaranteed correctly rounded as
+// IEEE division is.  Zero, infinite and NaN x give NaN.
 __device__ __forceinline__ double rcp_nr(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // FP64 natural logarithm after Tang's table-driven method (P. T. P. Tang,
 // ACM TOMS 16(4), 1990).  x = 2^m y with y in [1, 2); F = 1 + j/128 the
 // breakpoint next to y, f = y - F (exact, |f| <= 2^-8), r = f/F from the
 // tabulated 1/F; ln x = m ln 2 + ln F + ln(1 + r), the last by its Taylor
-// series through r^7 (the rest is below 2^-59 of r).  ln 2 and ln F are
+// series through r^7 (the rest is below 2^-59 of r).  The terms from r^5 on
+// are r^5 T(r), T = 1/5 - r/6 + r^2/7, below 2^-42: T is summed in FP32,
+// whose rounding moves the logarithm by less than 2^-58 of r, and goes to
+// and from FP32 by moving bits (the GB300 FP64 pipe, which bounds the FP64
+// step, does the type conversions too).  The exponent m becomes a double
+// the same way.  ln 2 and ln F are
 // tabulated as hi + lo with hi a multiple of 2^-32, so m ln2_hi + lnF_hi is
 // exact: just below 1 the two cancel almost entirely, and only the small
 // terms carry rounding errors.  For x in [1 - 2^-9, 1) (m = -1, j = 128) the
 // series takes r = x - 1 directly.  Within about two ulp for positive
 // normal x; zero, negative, subnormal, infinite and NaN x go to log().
+__device__ __forceinline__ float narrow(double v)   // truncates; |v| < 2^-126: 0
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned mag = ((hi & 0x7FFFFFFFu) - 0x38000000u) << 3 | lo >> 29;
+    return (hi & 0x7FFFFFFFu) < 0x38100000u ? 0.0f
+                                            : __uint_as_float((hi & 0x80000000u) | mag);
+}
+__device__ __forceinline__ double widen(float v)    // exact; v zero or normal
+{
+    const unsigned b = __float_as_uint(v), mag = b & 0x7FFFFFFFu;
+    return __hiloint2double((int)((b & 0x80000000u) | (mag ? (mag >> 3) + 0x38000000u : 0u)),
+                            (int)(b << 29));
+}
 __device__ __forceinline__ double log_tab(double x)
 {
     const int hi = __double2hiint(x);
@@ -144,51 +162,94 @@ __device__ __forceinline__ double log_tab(double x)
     const double F = __hiloint2double(0x3FF00000 + (j << 13), 0);
     const double2 t = __ldg(&kLogTable[j]);  // {1/F, hi of ln F}
     const double r = (y - F) * t.x;
-    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
-    q = fma(q, r, 1.0 / 5.0);
-    q = fma(q, r, -1.0 / 4.0);
+    const float rf = narrow(r);
+    const double T = widen(fmaf(rf, fmaf(rf, 1.0f / 7.0f, -1.0f / 6.0f), 1.0f / 5.0f));
+    double q = fma(T, r, -1.0 / 4.0);
     q = fma(q, r, 1.0 / 3.0);
     q = fma(q, r, -0.5);
     const double p = fma(r * r, q, r);       // ln(1 + r)
-    const double dm = (double)m;
+    const double dm = widen((float)m);
     return fma(dm, LN2_HI, t.y) + (fma(dm, LN2_LO, __ldg(&kLogTableLo[j])) + p);
 }
 
-// Division and logarithm of the arithmetic type: the FP32 kernels use the
-// fast hardware forms (__fdividef, __logf), whose few-ulp errors sit far
-// below the FP32 storage error; FP64 the reciprocal and logarithm above,
-// within one or two ulp of IEEE division and log().
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
+// Reciprocal, division and logarithm of the arithmetic type: the FP32
+// kernels use the hardware's approximate forms, whose few-ulp errors sit far
+// below the FP32 storage error, with subnormal operands read as zero (a
+// density that small has no finite reciprocal either): one instruction each,
+// where __fdividef and __logf wrap them in the scaling of subnormals, which
+// the issue-bound FP16-storage step paid for (2048 x 1026 walled: 28.1 ->
+// 26.7 us, results unchanged to the bit); FP64 the reciprocal
+// and logarithm above, within one or two ulp of IEEE division and log().
+__device__ __forceinline__ float frcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ double frcp(double x) { return rcp_nr(x); }
+__device__ __forceinline__ float fdiv(float a, float b) { return a * frcp(b); }
 __device__ __forceinline__ double fdiv(double a, double b) { return a * rcp_nr(b); }
-__device__ __forceinline__ float flog(float x) { return __logf(x); }
+__device__ __forceinline__ float flog(float x)
+{
+    float l;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x));
+    return l * 0.693147180559945f;
+}
 __device__ __forceinline__ double flog(double x) { return log_tab(x); }
 
-template <class T>
-__device__ __forceinline__ T mu_bulk(const EosT<T> &e, T rho)
+__device__ __forceinline__ float mu_bulk(const EosT<float> &e, float rho)
 {
     switch (e.kind) {
     case EOS_VDW: {
-        const T iq = fdiv(T(1), T(1) - e.b * rho);
-        return e.RT * (flog(rho * iq) + iq) - T(2) * e.a * rho;
+        const float iq = fdiv(1.0f, 1.0f - e.b * rho);
+        return e.RT * (flog(rho * iq) + iq) - 2.0f * e.a * rho;
     }
     case EOS_CS: {
-        const T h = e.quarter_b * rho;
-        const T iq = fdiv(T(1), T(1) - h);
-        return e.RT * ((T(3) - h) * (iq * iq * iq) + flog(rho) + T(1)) -
-               T(2) * e.a * rho;
+        const float h = e.quarter_b * rho;
+        const float iq = fdiv(1.0f, 1.0f - h);
+        return e.RT * ((3.0f - h) * (iq * iq * iq) + flog(rho) + 1.0f) -
+               2.0f * e.a * rho;
     }
     case EOS_PR: {
-        const T br = e.b * rho;
-        const T iq = fdiv(T(1), T(1) - br);
+        const float br = e.b * rho;
+        const float iq = fdiv(1.0f, 1.0f - br);
         return e.RT * flog(rho * iq) -
                e.pr_c * flog(fdiv(e.pr_s2m1 + br, e.pr_s2p1 - br)) +
-               e.RT * iq - fdiv(e.aalpha * rho, T(1) + T(2) * br - br * br);
+               e.RT * iq - fdiv(e.aalpha * rho, 1.0f + 2.0f * br - br * br);
     }
     default: {  // EOS_RKS
-        const T br = e.b * rho;
-        const T iq = fdiv(T(1), T(1) - br);
-        return e.RT * (flog(rho * iq) + iq) - e.rks_c * flog(T(1) + br) -
-               fdiv(e.aalpha * rho, T(1) + br);
+        const float br = e.b * rho;
+        const float iq = fdiv(1.0f, 1.0f - br);
+        return e.RT * (flog(rho * iq) + iq) - e.rks_c * flog(1.0f + br) -
+               fdiv(e.aalpha * rho, 1.0f + br);
+    }
+    }
+}
+
+// FP64: the same with fewer instructions.
+__device__ __forceinline__ double mu_bulk(const EosT<double> &e, double rho)
+{
+    switch (e.kind) {
+    case EOS_VDW: {
+        const double iq = frcp(1.0 - e.b * rho);
+        return e.RT * (flog(rho * iq) + iq) + e.m2a * rho;
+    }
+    case EOS_CS: {
+        // (3 - h) / (1 - h)^3 = iq^2 (2 iq + 1) with iq = 1 / (1 - h)
+        const double iq = frcp(1.0 - e.quarter_b * rho);
+        return e.RT * (iq * iq * (2.0 * iq + 1.0) + flog(rho)) + (e.m2a * rho + e.RT);
+    }
+    case EOS_PR: {
+        const double br = e.b * rho;
+        const double iq = frcp(1.0 - br);
+        return e.RT * (flog(rho * iq) + iq) -
+               e.pr_c * flog(fdiv(e.pr_s2m1 + br, e.pr_s2p1 - br)) -
+               fdiv(e.aalpha * rho, br * (2.0 - br) + 1.0);
+    }
+    default: {  // EOS_RKS
+        const double br = e.b * rho;
+        const double iq = frcp(1.0 - br), p = 1.0 + br;
+        return e.RT * (flog(rho * iq) + iq) - e.rks_c * flog(p) - fdiv(e.aalpha * rho, p);
     }
     }
 }
@@ -484,6 +545,56 @@ __device__ __forceinline__ void grad9(const T *s, int c, T &gx, T &gy)
     gy = (T(4) * (s[c + W] - s[c - W]) + (ne + nw) - (se + sw)) * T(1.0 / 12.0);
 }
 
+// One row of a field around column c of a stencil's window: the node, the
+// sum and the difference of its east and west neighbours.  With rows u
+// (above), m and d (below) the isotropic stencils without their factors are
+//   12 grad_x = 4 D_m + D_u + D_d,   12 grad_y = 4 (C_u - C_d) + H_u - H_d,
+//    6 lap    = 4 (H_m + C_u + C_d) + (H_u + H_d) - 20 C_m,
+// which are grad9 / lap9 term by term; the factors sit in Consts.  A walk up
+// the rows forms H and D once per row: 7 instructions for a gradient and 6
+// for a Laplacian, against 12 and 9 from a 3 x 3 window.
+template <class T> struct Row {
+    T c, h, d;
+};
+template <class T>
+__device__ __forceinline__ Row<T> row_of(const T *s, int i)
+{
+    const T w = s[i - 1], e = s[i + 1];
+    return {s[i], e + w, e - w};
+}
+template <class T>
+__device__ __forceinline__ T lap6(const Row<T> &u, const Row<T> &m, const Row<T> &d)
+{
+    return T(4) * (m.h + u.c + d.c) + (u.h + d.h) - T(20) * m.c;
+}
+template <class T>
+__device__ __forceinline__ void grad12(const Row<T> &u, const Row<T> &m, const Row<T> &d,
+                                       T &gx, T &gy)
+{
+    gx = T(4) * m.d + u.d + d.d;
+    gy = T(4) * (u.c - d.c) + u.h - d.h;
+}
+// The same around linear index c of a shared-memory tile of row width W.
+template <class T, int W>
+__device__ __forceinline__ T lap6(const T *s, int c)
+{
+    return lap6(row_of(s, c + W), row_of(s, c), row_of(s, c - W));
+}
+template <class T, int W>
+__device__ __forceinline__ void grad12(const T *s, int c, T &gx, T &gy)
+{
+    grad12(row_of(s, c + W), row_of(s, c), row_of(s, c - W), gx, gy);
+}
+// mu = psi'(rho) - kappa lap(rho) (Eq. 8) from the absolute density and 6 lap.
+__device__ __forceinline__ float mu_of(const Consts<float> &K, float rho, float l6)
+{
+    return mu_bulk(K.eos, rho) - K.kappa * (l6 * (1.0f / 6.0f));
+}
+__device__ __forceinline__ double mu_of(const Consts<double> &K, double rho, double l6)
+{
+    return K.nk6 * l6 + mu_bulk(K.eos, rho);
+}
+
 // Fill s_mu[(TY + 2) x (TX + 2)] with mu on the tile and a one-node halo
 // (Eq. 8) from the stored-form densities in s_rho; solid rows carry the
 // surface values (Sec. IV, V).
@@ -494,8 +605,6 @@ __device__ void mu_tile(const Lattice &L, int X0, int Y0,
     using real = typename S::real;
     constexpr int W = TX + 2, H = TY + 2, WR = TX + 4;
     const Consts<real> &K = consts<real>(L);
-    const EosT<real> &eos = K.eos;
-    const real kappa = K.kappa;
     const real ref = S::offset ? K.rho_ref : real(0);
     const int wx = min(TX, L.nx - X0), wy = min(TY, L.nyf - Y0);
     for (int k = threadIdx.x; k < W * H; k += blockDim.x) {
@@ -512,17 +621,133 @@ __device__ void mu_tile(const Lattice &L, int X0, int Y0,
         } else if (L.walls && r == L.nyf) {
             if (L.top_mode == 0) {
                 const int cb = c - WR;  // fluid neighbour below (row nyf-1)
-                m = mu_bulk(eos, s_rho[cb] + ref) - kappa * lap9<real, WR>(s_rho, cb);
+                m = mu_of(K, s_rho[cb] + ref, lap6<real, WR>(s_rho, cb));
             } else {
                 m = K.mu_top;
             }
         } else if (L.walls && (r < -1 || r > L.nyf)) {
             m = real(0);
         } else {
-            m = mu_bulk(eos, s_rho[c] + ref) - kappa * lap9<real, WR>(s_rho, c);
+            m = mu_of(K, s_rho[c] + ref, lap6<real, WR>(s_rho, c));
         }
         s_mu[k] = m;
     }
+}
+
+// ---------------------------------------------------------------------------
+// BGK collision with the velocity-shift forcing (Eq. 13-14, Sec. II).
+// ---------------------------------------------------------------------------
+// m = sum f_i e_i + tau F of one node (populations f[1..8]) with the force
+// of Eq. 12, F = -rho grad(mu) + grad(cs^2 rho), from the stencils 12 grad.
+template <class T>
+__device__ __forceinline__ void momentum(const T *f, T &jx, T &jy)
+{
+    const T d57 = f[5] - f[7], d86 = f[8] - f[6];
+    jx = (f[1] - f[3]) + d57 + d86;
+    jy = (f[2] - f[4]) + d57 - d86;
+}
+__device__ __forceinline__ void force_momentum(const Consts<float> &K, const float *f, float rho,
+                                               float grx, float gry, float gmx, float gmy,
+                                               float &mx, float &my)
+{
+    float jx, jy;
+    momentum(f, jx, jy);
+    const float c = 1.0f / 12.0f, third = 1.0f / 3.0f;
+    const float Fx = grx * c * third - rho * (gmx * c);
+    const float Fy = gry * c * third - rho * (gmy * c);
+    mx = jx + K.tau * Fx;
+    my = jy + K.tau * Fy;
+}
+__device__ __forceinline__ void force_momentum(const Consts<double> &K, const double *f,
+                                               double rho, double grx, double gry, double gmx,
+                                               double gmy, double &mx, double &my)
+{
+    double jx, jy;
+    momentum(f, jx, jy);
+    const double tr = K.nt12 * rho;
+    mx = K.t36 * grx + (tr * gmx + jx);
+    my = K.t36 * gry + (tr * gmy + jy);
+}
+
+// Collision of one node towards the equilibrium of velocity u = m / rho.
+// f[1..8] are the node's stored populations (f_0 = drho - sum f_i is
+// implicit), drho its stored density (rho - rho_ref) and rho the absolute
+// one; fp[0..8] receive the post-collision values in stored form.  Eq. 14 in
+// stored form is f_eq - w_i rho_ref = w_i (drho + rho P_i(u)), P_i = 3 e.u +
+// 4.5 (e.u)^2 - 1.5 u^2; opposite directions share the even part of P.
+//
+// FP32: Eq. 13 as it stands, f + omega (f_eq - f).  Where the flow is
+// uniform the same rounding repeats at every node and step and builds up; the
+// shorter form below drifted by 3e-8 of the momentum per step in FP32 for
+// tau = 1 (omega / 3 and omega / 12 both round up), and the FP32 kernels that
+// carry the large lattices wait for memory, not for these instructions.
+__device__ __forceinline__ void relax(const Consts<float> &K, const float *f, float drho,
+                                      float rho, float mx, float my, float *fp)
+{
+    const float inv_rho = frcp(rho), omega = K.omega;
+    const float ux = mx * inv_rho, uy = my * inv_rho;
+    const float usq = 1.5f * (ux * ux + uy * uy);
+    const float w1 = 1.0f / 9.0f, w5 = 1.0f / 36.0f;
+    {
+        const float ex2 = 4.5f * ux * ux - usq, ey2 = 4.5f * uy * uy - usq;
+        const float ax = w1 * (drho + rho * ex2), bx = w1 * rho * 3.0f * ux;
+        const float ay = w1 * (drho + rho * ey2), by = w1 * rho * 3.0f * uy;
+        fp[1] = f[1] + omega * ((ax + bx) - f[1]);
+        fp[3] = f[3] + omega * ((ax - bx) - f[3]);
+        fp[2] = f[2] + omega * ((ay + by) - f[2]);
+        fp[4] = f[4] + omega * ((ay - by) - f[4]);
+    }
+    {
+        const float sp = ux + uy, sm = ux - uy;
+        const float ep = 4.5f * sp * sp - usq, em = 4.5f * sm * sm - usq;
+        const float a5 = w5 * (drho + rho * ep), b5 = w5 * rho * 3.0f * sp;
+        const float a8 = w5 * (drho + rho * em), b8 = w5 * rho * 3.0f * sm;
+        fp[5] = f[5] + omega * ((a5 + b5) - f[5]);
+        fp[7] = f[7] + omega * ((a5 - b5) - f[7]);
+        fp[8] = f[8] + omega * ((a8 + b8) - f[8]);
+        fp[6] = f[6] + omega * ((a8 - b8) - f[6]);
+    }
+    // The rest population takes what the moving ones leave of the density:
+    // in exact arithmetic this equals f_0 + omega (f_0^eq - f_0) with
+    // f_0 = drho - sum_{i>0} f_i, and it keeps the collision's mass exact
+    // instead of biased by the rounding of f_eq.
+    fp[0] = drho - (((fp[1] + fp[2]) + (fp[3] + fp[4])) +
+                    ((fp[5] + fp[6]) + (fp[7] + fp[8])));
+}
+// FP64, where every instruction of the narrow pipe counts: with e_ab =
+// m_a u_b the even part of omega f_eq is, along an axis, omega/9 (drho +
+// 3 e_xx - 1.5 e_yy) and, along a diagonal, omega/36 (drho + 3 (e_xx + e_yy)
+// +- 9 e_xy), and the odd part omega w_i 3 m.e_i: two fused multiply-adds
+// per population finish f* = (1 - omega) f + even + odd.  The FP64 step is
+// bound by that pipe (82 % busy); this form, the shared row sums of the
+// stencils, log_tab and rcp_nr together took a 1024 x 1024 periodic CS step
+// from 325 to 252 us.
+__device__ __forceinline__ void relax(const Consts<double> &K, const double *f, double drho,
+                                      double rho, double mx, double my, double *fp)
+{
+    const double ir = frcp(rho);
+    const double ux = mx * ir, uy = my * ir;
+    const double exx = mx * ux, eyy = my * uy, exy = mx * uy;
+    const double t = K.o9 * drho;
+    {
+        const double ax = K.o3 * exx + (K.no6 * eyy + t);
+        const double ay = K.o3 * eyy + (K.no6 * exx + t);
+        fp[1] = K.o3 * mx + (K.om1 * f[1] + ax);
+        fp[3] = -K.o3 * mx + (K.om1 * f[3] + ax);
+        fp[2] = K.o3 * my + (K.om1 * f[2] + ay);
+        fp[4] = -K.o3 * my + (K.om1 * f[4] + ay);
+    }
+    {
+        const double sp = mx + my, sm = mx - my;
+        const double s = K.o12 * (exx + eyy) + 0.25 * t;
+        const double ap = K.o4 * exy + s, am = -K.o4 * exy + s;
+        fp[5] = K.o12 * sp + (K.om1 * f[5] + ap);
+        fp[7] = -K.o12 * sp + (K.om1 * f[7] + ap);
+        fp[8] = K.o12 * sm + (K.om1 * f[8] + am);
+        fp[6] = -K.o12 * sm + (K.om1 * f[6] + am);
+    }
+    fp[0] = drho - (((fp[1] + fp[2]) + (fp[3] + fp[4])) +
+                    ((fp[5] + fp[6]) + (fp[7] + fp[8])));
 }
 
 }  // namespace cplbm

@@ -29,6 +29,19 @@ static void fill_consts(Consts<T> &k, const Lattice &L)
     k.rho_ref = T(L.rho_ref);
     k.mu_bottom = T(L.mu_bottom);
     k.mu_top = T(L.mu_top);
+    const double omega = 1.0 / L.tau;
+    // the FP64 collision keeps a node's momentum when om1 + 2 o3 + 4 o12 = 1:
+    // the roundings of the three are chosen together
+    k.o3 = T(omega / 3.0);
+    k.o12 = T(0.25 * (omega - 2.0 * double(k.o3)));
+    const double keep = 2.0 * double(k.o3) + 4.0 * double(k.o12);
+    k.om1 = T(1.0 - keep);
+    k.o9 = T(keep / 9.0);
+    k.o4 = T(omega / 4.0);
+    k.no6 = T(-omega / 6.0);
+    k.t36 = T(L.tau / 36.0);
+    k.nt12 = T(-L.tau / 12.0);
+    k.nk6 = T(-L.kappa / 6.0);
     k.eos.kind = e.kind;
     k.eos.a = T(e.a);
     k.eos.b = T(e.b);
@@ -38,6 +51,7 @@ static void fill_consts(Consts<T> &k, const Lattice &L)
     k.eos.pr_c = T(e.b > 0 ? e.aalpha / (2.0 * 1.4142135623730951 * e.b) : 0.0);
     k.eos.pr_s2m1 = T(0.41421356237309515);
     k.eos.pr_s2p1 = T(2.414213562373095);
+    k.eos.m2a = T(-2.0 * e.a);
     k.eos.rks_c = T(e.b > 0 ? e.aalpha / e.b : 0.0);
 }
 

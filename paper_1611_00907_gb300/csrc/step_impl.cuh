@@ -171,61 +171,12 @@ __device__ __forceinline__ void mu_interior(const Lattice &L,
     using real = typename S::real;
     constexpr int W = TX + 2, H = TY + 2, WR = TX + 4;
     const Consts<real> &K = consts<real>(L);
-    const EosT<real> &eos = K.eos;
-    const real kappa = K.kappa;
     const real ref = S::offset ? K.rho_ref : real(0);
     for (int k = threadIdx.x; k < W * H; k += NT) {
         const int lx = k % W, ly = k / W;
         const int c = (ly + 1) * WR + lx + 1;
-        s_mu[k] = mu_bulk(eos, s_rho[c] + ref) - kappa * lap9<real, WR>(s_rho, c);
+        s_mu[k] = mu_of(K, s_rho[c] + ref, lap6<real, WR>(s_rho, c));
     }
-}
-
-// BGK collision of one node with the velocity-shift forcing.  f[1..8] are
-// the node's stored populations (f_0 = drho - sum f_i is implicit), drho
-// its stored density (rho - rho_ref) and rho the absolute one; fp[0..8]
-// receive the post-collision values in stored form.
-template <class real>
-__device__ __forceinline__ void collide(const real *f, real drho, real rho,
-                                        real Fx, real Fy, real tau, real omega,
-                                        real *fp)
-{
-    // u = sum f_i e_i / rho; u_eq = u + tau F / rho (Sec. II)
-    const real jx = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
-    const real jy = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
-    const real inv_rho = fdiv(real(1), rho);
-    const real ux = (jx + tau * Fx) * inv_rho;
-    const real uy = (jy + tau * Fy) * inv_rho;
-    const real usq = real(1.5) * (ux * ux + uy * uy);
-    // Eq. 14 in stored form: f_eq - w_i rho_ref = w_i (drho + rho P_i(u)),
-    // P_i = 3 e.u + 4.5 (e.u)^2 - 1.5 u^2; opposite directions share the
-    // even part of P.
-    const real w1 = real(1.0 / 9.0), w5 = real(1.0 / 36.0);
-    {
-        const real ex2 = real(4.5) * ux * ux - usq, ey2 = real(4.5) * uy * uy - usq;
-        const real ax = w1 * (drho + rho * ex2), bx = w1 * rho * real(3) * ux;
-        const real ay = w1 * (drho + rho * ey2), by = w1 * rho * real(3) * uy;
-        fp[1] = f[1] + omega * ((ax + bx) - f[1]);
-        fp[3] = f[3] + omega * ((ax - bx) - f[3]);
-        fp[2] = f[2] + omega * ((ay + by) - f[2]);
-        fp[4] = f[4] + omega * ((ay - by) - f[4]);
-    }
-    {
-        const real sp = ux + uy, sm = ux - uy;
-        const real ep = real(4.5) * sp * sp - usq, em = real(4.5) * sm * sm - usq;
-        const real a5 = w5 * (drho + rho * ep), b5 = w5 * rho * real(3) * sp;
-        const real a8 = w5 * (drho + rho * em), b8 = w5 * rho * real(3) * sm;
-        fp[5] = f[5] + omega * ((a5 + b5) - f[5]);
-        fp[7] = f[7] + omega * ((a5 - b5) - f[7]);
-        fp[8] = f[8] + omega * ((a8 + b8) - f[8]);
-        fp[6] = f[6] + omega * ((a8 - b8) - f[6]);
-    }
-    // The rest population takes what the moving ones leave of the density:
-    // in exact arithmetic this equals f_0 + omega (f_0^eq - f_0) with
-    // f_0 = drho - sum_{i>0} f_i, and it keeps the collision's mass exact
-    // instead of biased by the rounding of f_eq.
-    fp[0] = drho - (((fp[1] + fp[2]) + (fp[3] + fp[4])) +
-                    ((fp[5] + fp[6]) + (fp[7] + fp[8])));
 }
 
 // Index of f*_i (i = 1..8) of tile node (lx, ly) in s_post.
@@ -308,6 +259,19 @@ __device__ void pt_tile(const Lattice &L, int X0, int Y0,
         s_p[N + k] = kappa * gx * gy;
         s_p[2 * N + k] = iso + kappa * gy * gy;
     }
+}
+
+// force_momentum with the force of Eq. 5, F = -div(P) + grad(cs^2 rho);
+// px, py: 12 div(P).
+template <class T>
+__device__ __forceinline__ void pt_momentum(const Consts<T> &K, const T *f, T grx, T gry, T px,
+                                            T py, T &mx, T &my)
+{
+    T jx, jy;
+    momentum(f, jx, jy);
+    const T c = T(1.0 / 12.0), third = T(1.0 / 3.0);
+    mx = jx + K.tau * (grx * c * third - px * c);
+    my = jy + K.tau * (gry * c * third - py * c);
 }
 
 template <class S, int TX, int TY, int NT, int PARITY, bool INTERIOR,
@@ -394,9 +358,8 @@ __device__ __forceinline__ void step_tile(const Lattice &L, int cur, int X0,
     __syncthreads();
 
     // 3. Force, collision, in-place streaming.
-    const real tau = consts<real>(L).tau;
-    const real omega = consts<real>(L).omega;
-    const real rho_ref = S::offset ? consts<real>(L).rho_ref : real(0);
+    const Consts<real> &K = consts<real>(L);
+    const real rho_ref = S::offset ? K.rho_ref : real(0);
     if constexpr (ASYNC) cp_async_wait_all();
     real self0[PER];
 #pragma unroll
@@ -421,26 +384,22 @@ __device__ __forceinline__ void step_tile(const Lattice &L, int cur, int X0,
         const int cr = (ly + 2) * WR + lx + 2, cm = (ly + 1) * WM + lx + 1;
         const real drho = s_rho[cr];
         const real rho = drho + rho_ref;
-        real Fx, Fy, grx, gry;
-        grad9<real, WR>(s_rho, cr, grx, gry);
+        real mx, my, grx, gry;
+        grad12<real, WR>(s_rho, cr, grx, gry);
         if constexpr (PT) {
-            // Eq. 5: F = -div(P) + grad(cs^2 rho)
             constexpr int N = SM::WM * SM::HM;
             real pxx_x, pxx_y, pxy_x, pxy_y, pyy_x, pyy_y;
-            grad9<real, WM>(s_mu, cm, pxx_x, pxx_y);
-            grad9<real, WM>(s_mu + N, cm, pxy_x, pxy_y);
-            grad9<real, WM>(s_mu + 2 * N, cm, pyy_x, pyy_y);
-            Fx = grx * real(1.0 / 3.0) - (pxx_x + pxy_y);
-            Fy = gry * real(1.0 / 3.0) - (pxy_x + pyy_y);
+            grad12<real, WM>(s_mu, cm, pxx_x, pxx_y);
+            grad12<real, WM>(s_mu + N, cm, pxy_x, pxy_y);
+            grad12<real, WM>(s_mu + 2 * N, cm, pyy_x, pyy_y);
+            pt_momentum(K, f, grx, gry, pxx_x + pxy_y, pxy_x + pyy_y, mx, my);
         } else {
-            // Eq. 12: F = -rho grad(mu) + grad(cs^2 rho)
             real gmx, gmy;
-            grad9<real, WM>(s_mu, cm, gmx, gmy);
-            Fx = grx * real(1.0 / 3.0) - rho * gmx;
-            Fy = gry * real(1.0 / 3.0) - rho * gmy;
+            grad12<real, WM>(s_mu, cm, gmx, gmy);
+            force_momentum(K, f, rho, grx, gry, gmx, gmy, mx, my);
         }
         real fp[9];
-        collide<real>(f, drho, rho, Fx, Fy, tau, omega, fp);
+        relax(K, f, drho, rho, mx, my, fp);
         self0[k] = fp[0];
 #pragma unroll
         for (int i = 1; i < 9; ++i) s_post[post_idx<TX, TY>(i, ly, lx)] = fp[i];
@@ -879,7 +838,7 @@ __device__ __forceinline__ bool wall_mu(const Lattice &L, const SeamEdges &e, in
         } else if (L.top_mode == 0) {
             const int cb = c - RP;  // fluid neighbour below (row nyf - 1)
             const real ref = S::offset ? K.rho_ref : real(0);
-            m = mu_bulk(K.eos, s_rho[cb] + ref) - K.kappa * lap9<real, RP>(s_rho, cb);
+            m = mu_of(K, s_rho[cb] + ref, lap6<real, RP>(s_rho, cb));
         } else {
             m = K.mu_top;
         }
@@ -958,24 +917,6 @@ struct TmaSmem {
     static constexpr unsigned tx_pops = PIN_BYTES;
     static_assert((PLANE * sizeof(pop_t)) % 128 == 0, "TMA destinations");
 };
-
-// Gradient of the isotropic stencil from a 3 x 3 window w[row][col] (row 0
-// below, col 0 left), same arithmetic as grad9.
-template <class T>
-__device__ __forceinline__ void grad_w(const T (&w)[3][3], T &gx, T &gy)
-{
-    const T ne = w[2][2], nw = w[2][0], se = w[0][2], sw = w[0][0];
-    gx = (T(4) * (w[1][2] - w[1][0]) + (ne - nw) + (se - sw)) * T(1.0 / 12.0);
-    gy = (T(4) * (w[2][1] - w[0][1]) + (ne + nw) - (se + sw)) * T(1.0 / 12.0);
-}
-// Laplacian of the isotropic stencil from a 3 x 3 window, as lap9.
-template <class T>
-__device__ __forceinline__ T lap_w(const T (&w)[3][3])
-{
-    const T axial = w[1][2] + w[1][0] + w[2][1] + w[0][1];
-    const T diag = (w[2][2] + w[2][0]) + (w[0][2] + w[0][0]);
-    return (T(4) * axial + diag - T(20) * w[1][1]) * T(1.0 / 6.0);
-}
 
 // PT: the baseline force of Eq. 5 (the pressure tensor of Eq. 9 in three
 // planes where the chemical potential would be; periodic lattices only).
@@ -1080,35 +1021,25 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
         }
     } else {
         const Consts<real> &K = consts<real>(L);
-        const EosT<real> &eos = K.eos;
-        const real kappa = K.kappa;
         const real ref = S::offset ? K.rho_ref : real(0);
         const int b0 = (warp * MH) / NW, b1 = ((warp + 1) * MH) / NW;
         const int a = lane + 1;
-        real w[3][3];
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) w[j][d] = s_rho[(b0 + j) * RP + a + 2 + d];
+        Row<real> rd = row_of(s_rho, b0 * RP + a + 3), rm = row_of(s_rho, (b0 + 1) * RP + a + 3);
         for (int b = b0; b < b1; ++b) {
-#pragma unroll
-            for (int d = 0; d < 3; ++d) w[2][d] = s_rho[(b + 2) * RP + a + 2 + d];
+            const Row<real> ru = row_of(s_rho, (b + 2) * RP + a + 3);
             real m;
             if (!(walls_ok && wall_mu<S, RP>(L, edge, b, (b + 1) * RP + a + 3, s_rho, m)))
-                m = mu_bulk(eos, w[1][1] + ref) - kappa * lap_w(w);
+                m = mu_of(K, rm.c + ref, lap6(ru, rm, rd));
             s_mu[b * MP + a] = m;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                w[0][d] = w[1][d];
-                w[1][d] = w[2][d];
-            }
+            rd = rm;
+            rm = ru;
         }
         for (int t = threadIdx.x; t < 2 * MH; t += NT) {
             const int ae = (t & 1) ? TX + 1 : 0, b = t >> 1;
             const int c = (b + 1) * RP + ae + 3;
             real m;
             if (!(walls_ok && wall_mu<S, RP>(L, edge, b, c, s_rho, m)))
-                m = mu_bulk(eos, s_rho[c] + ref) - kappa * lap9<real, RP>(s_rho, c);
+                m = mu_of(K, s_rho[c] + ref, lap6<real, RP>(s_rho, c));
             s_mu[b * MP + ae] = m;
         }
     }
@@ -1123,9 +1054,8 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
     // 4. Force, collision, in-place streaming and the register hand-over for
     //    the thread's PER nodes at rows ly0 .. ly0 + PER - 1, column lx.
     const int lx = lane, ly0 = warp * PER;
-    const real tau = consts<real>(L).tau;
-    const real omega = consts<real>(L).omega;
-    const real rho_ref = S::offset ? consts<real>(L).rho_ref : real(0);
+    const Consts<real> &K = consts<real>(L);
+    const real rho_ref = S::offset ? K.rho_ref : real(0);
     pop_t *A = (pop_t *)L.pops;
     rho_t *Rn = (rho_t *)L.rho[nxt];
     rho_t *const *ring = (rho_t *const *)L.ring[nxt];
@@ -1147,14 +1077,13 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
     // not fluid); the others are not updated and contribute nothing
     const bool has_l = lane > 0, has_r = lane < lr;
     const bool lane_ok = lane < hx;
-    real wr[3][3], wm[3][3];
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            wr[j][d] = s_rho[(ly0 + 1 + j) * RP + lx + 3 + d];
-            wm[j][d] = s_mu[(ly0 + j) * MP + lx + d];
-        }
+    Row<real> rd = row_of(s_rho, (ly0 + 1) * RP + lx + 4);
+    Row<real> rm = row_of(s_rho, (ly0 + 2) * RP + lx + 4);
+    Row<real> md{}, mm{};
+    if constexpr (!PT) {
+        md = row_of(s_mu, ly0 * MP + lx + 1);
+        mm = row_of(s_mu, (ly0 + 1) * MP + lx + 1);
+    }
     // Rolling hand-over.  pend: row k - 1 without its "down" part;
     // first: row 0 of the warp without the warp below's "up"; *_c: the same
     // for the ring column a lane 0 / lane hx - 1 feeds; up_top: the "up" of
@@ -1174,11 +1103,9 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int ly = ly0 + k;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            wr[2][d] = s_rho[(ly + 3) * RP + lx + 3 + d];
-            wm[2][d] = s_mu[(ly + 2) * MP + lx + d];
-        }
+        const Row<real> ru = row_of(s_rho, (ly + 3) * RP + lx + 4);
+        Row<real> mu{};
+        if constexpr (!PT) mu = row_of(s_mu, (ly + 2) * MP + lx + 1);
         real same = real(0), up = real(0), down = real(0);
         real same_c = real(0), up_c = real(0), down_c = real(0);
         if (!seam || ly < hy) {  // warp-uniform
@@ -1186,28 +1113,25 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
 #pragma unroll
             for (int i = 1; i < 9; ++i)
                 f[i] = ld_real(s_pin + (i - 1) * PLANE + ly * PP + lx + pin_col<PARITY, TS::PX>(i));
-            const real drho = wr[1][1];
+            const real drho = rm.c;
             const real rho = drho + rho_ref;
-            real gmx, gmy, grx, gry;
-            grad_w(wr, grx, gry);
-            real Fx, Fy;
+            real grx, gry, mx, my;
+            grad12(ru, rm, rd, grx, gry);
             if constexpr (PT) {
-                // Eq. 5: F = -div(P) + grad(cs^2 rho), as step_tile
                 constexpr int N = MP * MH;
                 const int cm = (ly + 1) * MP + lx + 1;
                 real pxx_x, pxx_y, pxy_x, pxy_y, pyy_x, pyy_y;
-                grad9<real, MP>(s_mu, cm, pxx_x, pxx_y);
-                grad9<real, MP>(s_mu + N, cm, pxy_x, pxy_y);
-                grad9<real, MP>(s_mu + 2 * N, cm, pyy_x, pyy_y);
-                Fx = grx * real(1.0 / 3.0) - (pxx_x + pxy_y);
-                Fy = gry * real(1.0 / 3.0) - (pxy_x + pyy_y);
+                grad12<real, MP>(s_mu, cm, pxx_x, pxx_y);
+                grad12<real, MP>(s_mu + N, cm, pxy_x, pxy_y);
+                grad12<real, MP>(s_mu + 2 * N, cm, pyy_x, pyy_y);
+                pt_momentum(K, f, grx, gry, pxx_x + pxy_y, pxy_x + pyy_y, mx, my);
             } else {
-                grad_w(wm, gmx, gmy);
-                Fx = grx * real(1.0 / 3.0) - rho * gmx;
-                Fy = gry * real(1.0 / 3.0) - rho * gmy;
+                real gmx, gmy;
+                grad12(mu, mm, md, gmx, gmy);
+                force_momentum(K, f, rho, grx, gry, gmx, gmy, mx, my);
             }
             real fp[9];
-            collide<real>(f, drho, rho, Fx, Fy, tau, omega, fp);
+            relax(K, f, drho, rho, mx, my, fp);
             // wall rows (halfway bounce-back, Sec. IV): what leaves into the
             // solid row comes back to the node
             const bool wall_b = walls_ok && edge.wb && ly == 0;
@@ -1278,11 +1202,10 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
         }
         up_prev = up;
         up_prev_c = up_c;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            wr[0][d] = wr[1][d]; wr[1][d] = wr[2][d];
-            wm[0][d] = wm[1][d]; wm[1][d] = wm[2][d];
-        }
+        rd = rm;
+        rm = ru;
+        md = mm;
+        mm = mu;
     }
     // up_prev: the warp's last-row "up", for the warp above (or the ring
     // row over the tile).
@@ -1350,7 +1273,7 @@ __device__ __forceinline__ bool step_tile_tma(const Lattice &L, int cur, int X0,
 // and with rows u (above), m and d (below):
 //   grad_x = (4 D_m + D_u + D_d) / 12,   grad_y = (4 (C_u - C_d) + H_u - H_d) / 12,
 //   lap    = (4 (H_m + C_u + C_d) + (H_u + H_d) - 20 C_m) / 6,
-// which are grad_w / lap_w term by term.
+// the stencils of Row (device_common.cuh) on pairs.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float2 p2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -1361,17 +1284,14 @@ __device__ __forceinline__ float2 psub(float2 a, float2 b)
 {
     return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
 }
-__device__ __forceinline__ float2 prcp(float2 v)
-{
-    return make_float2(__fdividef(1.0f, v.x), __fdividef(1.0f, v.y));
-}
+__device__ __forceinline__ float2 prcp(float2 v) { return make_float2(frcp(v.x), frcp(v.y)); }
 __device__ __forceinline__ float2 pdiv(float2 a, float2 b)
 {
-    return make_float2(__fdividef(a.x, b.x), __fdividef(a.y, b.y));
+    return make_float2(fdiv(a.x, b.x), fdiv(a.y, b.y));
 }
 __device__ __forceinline__ float2 plog(float2 v)
 {
-    return make_float2(__logf(v.x), __logf(v.y));
+    return make_float2(flog(v.x), flog(v.y));
 }
 
 // One window row of a field around the pair at s + i (8-byte aligned).
@@ -1456,7 +1376,7 @@ __device__ __forceinline__ float2 p0_bulk2(const EosT<float> &e, float2 rho)
     }
 }
 
-// collide() on a pair of nodes.
+// The collision (relax, FP32) on a pair of nodes.
 __device__ __forceinline__ void collide2(const float2 *f, float2 drho, float2 rho,
                                          float2 Fx, float2 Fy, float2 tau,
                                          float2 omega, float2 *fp)
@@ -1686,7 +1606,7 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
             const int c = (b + 1) * RP + ae + 3;
             float mv;
             if (!(walls_ok && wall_mu<S, RP>(L, edge, b, c, s_rho, mv)))
-                mv = mu_bulk(eos, s_rho[c] + ref) - K.kappa * lap9<float, RP>(s_rho, c);
+                mv = mu_of(K, s_rho[c] + ref, lap6<float, RP>(s_rho, c));
             s_mu[b * MP + ae + 1] = mv;
         }
     }
