@@ -88,7 +88,9 @@ typedef struct {
 
 /* Allocate a context and its device state for cfg.  *out receives the
  * context (NULL on error).  Device memory per lattice node: 8 distributions
- * in the storage type plus three densities. */
+ * in the storage type plus three densities; lattices that lbm_step can keep
+ * on the chip (below) take 36 more values per node for the words their
+ * tiles exchange. */
 lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out);
 
 /* Select the equation of state (Sec. III): a, b, R as in Eqs. 16, 19, 22,
@@ -107,7 +109,9 @@ lbm_status lbm_set_wall_mu(lbm_ctx *ctx, double mu_bottom, int top_mode,
                            double mu_top);
 
 /* Tile shape of the fused step kernel: tx x ty fluid nodes per CTA, one of
- * 32x16, 32x24, 32x32, 64x16, 64x32 (LBM_ERR_ARG otherwise).  The shape
+ * 32x16, 32x24, 32x32, 64x16, 64x32 (LBM_ERR_ARG otherwise).  Choosing one
+ * also makes lbm_step take that kernel for every step, on small lattices too
+ * (lbm_autotune chooses between the two).  The shape
  * changes speed, and in FP32 arithmetic the rounding order of some sums,
  * not the method.  May be called at any time.  Default: 64x16 (two nodes
  * per lane) for FP32 arithmetic, 32x32 for FP64. */
@@ -116,7 +120,9 @@ lbm_status lbm_get_tile(const lbm_ctx *ctx, int *tx, int *ty);
 
 /* Time nsteps (rounded up to an even count >= 2) steps of each compiled
  * tile shape of the force model in use (lbm_set_force_model) on the
- * context's own lattice, keep the fastest, and restore
+ * context's own lattice, and of the on-chip steps of a small lattice
+ * (lbm_step; *tx, *ty then receive the default shape), keep the fastest, and
+ * restore
  * the state exactly as it was (the step counter included).  Allocates one
  * temporary copy of the state.  *tx, *ty (may be NULL) receive the shape. */
 lbm_status lbm_autotune(lbm_ctx *ctx, int nsteps, int *tx, int *ty);
@@ -142,8 +148,12 @@ lbm_status lbm_init(lbm_ctx *ctx, const double *rho, const double *ux,
 
 /* Queue nsteps (>= 0) time steps (Sec. II: density, Eq. 8, Eq. 12, the
  * BGK collision of Eq. 13-14 and streaming, with the wall rule of Sec. IV)
- * on the context's stream.  Returns without waiting for the GPU.  Blocks of
- * 16 steps replay a CUDA graph captured on a private stream at the first
+ * on the context's stream.  Returns without waiting for the GPU.  Four steps
+ * or more of a lattice whose state fits the shared memory of all SMs together
+ * (FP64 up to about 270 000 nodes, FP32 storage about 500 000; not FP16, the
+ * pressure-tensor force or a chosen tile shape) run as one cooperative launch
+ * that keeps the state there; such launches follow one another on a device.
+ * Otherwise blocks of 16 steps replay a CUDA graph captured on a private stream at the first
  * such call (and again after any change of tile shape, physics, force
  * model or wait limit); while the context's stream is being captured by
  * the caller, every step is a plain launch that joins the caller's graph. */
@@ -215,7 +225,10 @@ lbm_status lbm_batch_create(const lbm_instance *inst, int count, int precision,
  * number of steps (the in-place order is then the natural one). */
 lbm_status lbm_batch_init(lbm_batch *b, int index, const double *rho,
                           const double *ux, const double *uy, int on_device);
-/* Queue nsteps steps of every active lattice; all must be initialised. */
+/* Queue nsteps steps of every active lattice; all must be initialised.  Four
+ * steps or more of lattices that together fit the shared memory of all SMs
+ * run on the chip, as lbm_step's (not after lbm_batch_set_tile or
+ * lbm_batch_schedule with a schedule). */
 lbm_status lbm_batch_step(lbm_batch *b, int nsteps);
 /* Take lattice `index` out of the batched launch (active = 0) or put it
  * back (active = 1).  An inactive lattice keeps its state and step count and

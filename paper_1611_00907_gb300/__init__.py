@@ -179,7 +179,8 @@ class Simulation:
         return self
 
     def set_tile(self, tx, ty):
-        """Tile shape of the step kernel (speed only; results unchanged)."""
+        """Tile shape of the step kernel (speed only; results unchanged).  A
+        small lattice then takes that kernel instead of its on-chip steps."""
         self._check(self._lib.lbm_set_tile(self._ctx, int(tx), int(ty)))
         return self
 

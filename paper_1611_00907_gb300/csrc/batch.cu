@@ -60,6 +60,14 @@ struct lbm_batch {
     long long t = 0;
     long long nodes = 0;
     cudaGraphExec_t exec = nullptr;  // GRAPH_STEPS steps from an even step
+    // small batches: blocks of steps with the states in shared memory
+    // (resident.cu), unless the caller has chosen a tile shape or schedule
+    bool tiles_chosen = false;
+    ResidentPlan plan;             // of the active lattices; empty: none
+    ResidentTile *d_tiles = nullptr;
+    void *d_xchg = nullptr;
+    size_t xchg_cap = 0;
+    unsigned xchg_tag = 1;
     std::string err;
 };
 
@@ -94,11 +102,74 @@ void drop_graph(lbm_batch *b)
     b->exec = nullptr;
 }
 
+// Cut the active lattices for the resident steps, when all of them together
+// fit the GPU's shared memory: their tiles, and the exchange words that
+// their descriptors (copies in lats) point to.
+lbm_status plan_resident(lbm_batch *b, std::vector<Lattice> &lats)
+{
+    std::vector<Lattice> on;
+    std::vector<int> index;
+    for (size_t i = 0; i < lats.size(); ++i)
+        if (b->active[i]) {
+            on.push_back(lats[i]);
+            index.push_back((int)i);
+        }
+    ResidentPlan p;
+    if (on.empty() || !resident_plan(on.data(), (int)on.size(), b->device, &p)) return LBM_OK;
+    size_t need = 0;
+    for (const Lattice &L : on) need += xchg_bytes(L);
+    if (need > b->xchg_cap) {
+        dev_free(b->d_xchg);
+        b->d_xchg = nullptr;
+        b->xchg_cap = 0;
+        BCUDA(b, dev_alloc(&b->d_xchg, need));
+        b->xchg_cap = need;
+        // zero is no step's tag; words of an earlier cut carry older tags
+        BCUDA(b, cudaMemsetAsync(b->d_xchg, 0, need, b->stream));
+    }
+    char *x = (char *)b->d_xchg;
+    for (int i : index) {
+        lats[i].xchg = x;
+#ifdef CPLBM_CHECK_BOUNDS
+        lats[i].b_xchg = (long long)xchg_bytes(lats[i]);
+#endif
+        x += xchg_bytes(lats[i]);
+    }
+    for (ResidentTile &t : p.tiles) t.inst = index[t.inst];
+    dev_free(b->d_tiles);
+    b->d_tiles = nullptr;
+    BCUDA(b, dev_alloc((void **)&b->d_tiles, p.tiles.size() * sizeof(ResidentTile)));
+    BCUDA(b, cudaMemcpy(b->d_tiles, p.tiles.data(), p.tiles.size() * sizeof(ResidentTile),
+                        cudaMemcpyHostToDevice));
+    b->plan = std::move(p);
+    return LBM_OK;
+}
+
+// Steps queued as resident launches (0 when they do not apply).
+int resident_steps(lbm_batch *b, int left)
+{
+    int done = 0;
+    while (!b->plan.tiles.empty() && left - done >= RESIDENT_MIN) {
+        const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
+        if (launch_resident(b->plan, nullptr, b->d_lats, b->d_tiles, n, (int)(b->t & 1),
+                            b->xchg_tag, b->stream) != cudaSuccess) {
+            cudaGetLastError();  // no co-resident launch here: the tile kernels
+            b->plan = ResidentPlan{};
+            break;
+        }
+        b->xchg_tag += (unsigned)n;
+        b->t += n;
+        done += n;
+    }
+    return done;
+}
+
 // Apply the batch tile shape to every lattice and rebuild the device copies
 // of the descriptors, the work list and the groups' tensor maps.
 lbm_status rebuild(lbm_batch *b)
 {
     drop_graph(b);
+    b->plan = ResidentPlan{};
     const int n = (int)b->inst.size();
     std::vector<Lattice> lats;
     std::vector<WorkItem> items;
@@ -194,6 +265,10 @@ lbm_status rebuild(lbm_batch *b)
             grp.n_uniform = k;
         }
         b->groups.push_back(std::move(grp));
+    }
+    if (!b->tiles_chosen && b->inst[0]->use_tma) {
+        lbm_status st = plan_resident(b, lats);
+        if (st != LBM_OK) return st;
     }
     dev_free(b->d_lats);
     dev_free(b->d_items);
@@ -359,7 +434,7 @@ lbm_status lbm_batch_create(const lbm_instance *inst, int count, int precision,
         lbm_config cfg{q.nx, q.ny, q.walls, q.tau, q.kappa, q.rho_ref, precision,
                        (void *)b->stream, device};
         lbm_ctx *c = nullptr;
-        st = lbm_create(&cfg, &c);
+        st = ctx_create(&cfg, false, &c);
         if (st != LBM_OK) {
             bfail(b, st, "lattice %d: %s", i, lbm_last_error(nullptr));
             break;
@@ -409,6 +484,7 @@ lbm_status lbm_batch_step(lbm_batch *b, int nsteps)
     const long long t0 = b->t;
     int left = b->n_items > 0 ? nsteps : 0;  // nothing to launch: time only
     lbm_status st = LBM_OK;
+    left -= resident_steps(b, left);
     if (left > 0 && (b->t & 1)) {
         st = launch_one(b);
         --left;
@@ -492,6 +568,7 @@ lbm_status lbm_batch_set_tile(lbm_batch *b, int tx, int ty)
     }
     b->tx = tx;
     b->ty = ty;
+    b->tiles_chosen = true;
     return rebuild(b);
 }
 
@@ -504,6 +581,10 @@ lbm_status lbm_batch_schedule(lbm_batch *b, int items_per_cta, int *current)
     if (items_per_cta >= 0 && items_per_cta != b->per_cta) {
         b->per_cta = items_per_cta;
         drop_graph(b);  // the captured launches carry the old grid
+    }
+    if (items_per_cta >= 0) {  // the caller wants the tile kernels
+        b->tiles_chosen = true;
+        b->plan = ResidentPlan{};
     }
     if (current) *current = b->per_cta;
     return LBM_OK;
@@ -540,10 +621,13 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
     // configurations: every tile shape with a grid row per lattice (groups of
     // one geometry) or 1, 2 or 4 work items per CTA
     const int per[4] = {0, 1, 2, 4};
+    // and last (k == 4 n) the resident steps, on the default shape
     auto restore = [&](int k) -> lbm_status {
-        b->tx = sx[k / 4];
-        b->ty = sy[k / 4];
-        b->per_cta = per[k % 4];
+        const bool stay = k == 4 * n;
+        b->tiles_chosen = !stay;
+        b->tx = stay ? 32 : sx[k / 4];
+        b->ty = stay ? 32 : sy[k / 4];
+        b->per_cta = stay ? 0 : per[k % 4];
         lbm_status s2 = rebuild(b);
         for (size_t i = 0; i < b->inst.size() && s2 == LBM_OK; ++i)
             s2 = ctx_snapshot(b->inst[i], snaps[i], false);
@@ -551,11 +635,13 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
         for (size_t i = 0; i < b->inst.size(); ++i) b->inst[i]->t = tsave[i];
         return s2;
     };
-    for (int k = 0; k < 4 * n && st == LBM_OK; ++k) {
-        if (!step_shape_supported(b->precision, sx[k / 4], sy[k / 4])) continue;
+    for (int k = 0; k <= 4 * n && st == LBM_OK; ++k) {
+        if (k < 4 * n && !step_shape_supported(b->precision, sx[k / 4], sy[k / 4])) continue;
         st = restore(k);
         if (st != LBM_OK) break;
-        if (per[k % 4] == 0) {  // the same launches as one item per CTA otherwise
+        if (k == 4 * n) {
+            if (b->plan.tiles.empty()) continue;
+        } else if (per[k % 4] == 0) {  // the same launches as one item per CTA otherwise
             bool any = false;
             for (const Group &g : b->groups) any = any || g.n_uniform > 0;
             if (!any) continue;
@@ -566,7 +652,8 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
             st = bfail(b, LBM_ERR_CUDA, "event record");
             break;
         }
-        for (int s = 0; s < nsteps && st == LBM_OK; ++s) st = launch_one(b);
+        for (int s = resident_steps(b, nsteps); s < nsteps && st == LBM_OK; ++s)
+            st = launch_one(b);
         float ms = 0.f;
         if (st == LBM_OK && (cudaEventRecord(e1, b->stream) != cudaSuccess ||
                              cudaEventSynchronize(e1) != cudaSuccess ||
@@ -611,6 +698,8 @@ void lbm_batch_destroy(lbm_batch *b)
     for (lbm_ctx *c : b->inst) lbm_destroy(c);
     dev_free(b->d_lats);
     dev_free(b->d_items);
+    dev_free(b->d_tiles);
+    dev_free(b->d_xchg);
     for (cudaStream_t st : b->aux) cudaStreamDestroy(st);
     for (cudaEvent_t ev : b->joins) cudaEventDestroy(ev);
     if (b->fork) cudaEventDestroy(b->fork);

@@ -263,6 +263,7 @@ void free_all(lbm_ctx *c)
     dev_free(c->d_prev);
     dev_free(c->d_tmp);
     dev_free(c->d_err);
+    dev_free(L.xchg);
 }
 
 // Tensor maps for the current tile shape (the TMA path is skipped when they
@@ -305,6 +306,32 @@ cudaError_t launch_one_step(lbm_ctx *c, cudaStream_t s)
     const int p = (int)(c->t & 1);
     return c->force_model == 1 ? launch_step_pt(c->L, p, p, s, &c->maps)
                                : launch_step(c->L, p, p, s, &c->maps);
+}
+
+// Steps queued as resident launches (0 when they do not apply).
+int resident_steps(lbm_ctx *c, int left)
+{
+    if (!c->resident || c->force_model != 0 || left < RESIDENT_MIN) return 0;
+    // a caller's capture takes plain launches: the words' tags are good for
+    // one run only
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (c->stream && (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess ||
+                      cs != cudaStreamCaptureStatusNone))
+        return 0;
+    int done = 0;
+    while (left - done >= RESIDENT_MIN) {
+        const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
+        if (launch_resident(c->plan, &c->L, nullptr, nullptr, n, (int)(c->t & 1), c->xchg_tag,
+                            c->stream) != cudaSuccess) {
+            cudaGetLastError();  // no co-resident launch here: the tile kernels
+            c->resident = false;
+            break;
+        }
+        c->xchg_tag += (unsigned)n;
+        c->t += n;
+        done += n;
+    }
+    return done;
 }
 
 // The graph of STEP_GRAPH_STEPS steps from an even step, captured on a
@@ -373,9 +400,8 @@ double host_alpha(int kind, double Tr, double omega)
 void set_global_error(const char *msg) { g_err = msg; }
 }  // namespace cplbm
 
-extern "C" {
-
-lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
+namespace cplbm {
+lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
 {
     if (out) *out = nullptr;
     if (!cfg || !out) return fail(nullptr, LBM_ERR_ARG, "null argument");
@@ -447,6 +473,18 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
     alloc((void **)&c->d_bad, sizeof(int));
     alloc((void **)&c->d_prev, (size_t)L.nx * L.ny * sizeof(double));
     alloc((void **)&c->d_err, sizeof(int));
+    const char *no_tma = getenv("CPLBM_NO_TMA");
+    c->use_tma = !(no_tma && no_tma[0] == '1');
+    if (alone && c->use_tma && st == LBM_OK && resident_plan(&L, 1, c->device, &c->plan)) {
+        alloc(&L.xchg, xchg_bytes(L));
+        c->resident = st == LBM_OK;
+#ifdef CPLBM_CHECK_BOUNDS
+        L.b_xchg = (long long)xchg_bytes(L);
+#endif
+        // zero is no step's tag
+        if (c->resident && cudaMemsetAsync(L.xchg, 0, xchg_bytes(L), c->stream) != cudaSuccess)
+            st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
+    }
     if (st == LBM_OK && cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess)
         st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
     if (st != LBM_OK) {
@@ -456,11 +494,17 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
     }
     L.err = c->d_err;
     L.wait_cycles = WAIT_CYCLES_DEFAULT;
-    const char *no_tma = getenv("CPLBM_NO_TMA");
-    c->use_tma = !(no_tma && no_tma[0] == '1');
     refresh_maps(c);
     *out = c;
     return LBM_OK;
+}
+}  // namespace cplbm
+
+extern "C" {
+
+lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out)
+{
+    return ctx_create(cfg, true, out);
 }
 
 lbm_status lbm_eos_critical(int eos, double a, double b, double R, double *Tc,
@@ -582,10 +626,9 @@ lbm_status lbm_eos_info(const lbm_ctx *c, double *T, double *alpha,
     return LBM_OK;
 }
 
-lbm_status lbm_set_tile(lbm_ctx *c, int tx, int ty)
+namespace {
+lbm_status change_tile(lbm_ctx *c, int tx, int ty)
 {
-    CPLBM_TRACE("lbm_set_tile");
-    if (!c) return fail(nullptr, LBM_ERR_ARG, "null context");
     if (!step_shape_supported(c->L.precision, tx, ty))
         return fail(c, LBM_ERR_ARG, "no step kernel for tile %d x %d", tx, ty);
     if (c->force_model == 1 && !pt_shape_supported(c->L.precision, tx, ty))
@@ -608,6 +651,16 @@ lbm_status lbm_set_tile(lbm_ctx *c, int tx, int ty)
     c->L.ty = ty;
     refresh_maps(c);
     return LBM_OK;
+}
+}  // namespace
+
+lbm_status lbm_set_tile(lbm_ctx *c, int tx, int ty)
+{
+    CPLBM_TRACE("lbm_set_tile");
+    if (!c) return fail(nullptr, LBM_ERR_ARG, "null context");
+    const lbm_status st = change_tile(c, tx, ty);
+    if (st == LBM_OK) c->resident = false;  // the caller wants the tile kernels
+    return st;
 }
 
 namespace {
@@ -653,11 +706,15 @@ lbm_status lbm_autotune(lbm_ctx *c, int nsteps, int *best_tx, int *best_ty)
     const long long t0 = c->t;
     int best = -1;
     float best_ms = 0.f;
+    // where the lattice has a plan for the resident steps they are timed
+    // beside the shapes (as shape index n, on the default shape)
+    const bool can_stay = !c->plan.tiles.empty() && c->force_model == 0;
+    if (can_stay && n < 16) step_default_shape(L.precision, &tx[n], &ty[n]);
     lbm_status st = snapshot(c, snap, true);
     cudaError_t e = cudaSuccess;
     if (st == LBM_OK) e = cudaEventCreate(&e0);
     if (st == LBM_OK && e == cudaSuccess) e = cudaEventCreate(&e1);
-    for (int k = 0; k < n && st == LBM_OK && e == cudaSuccess; ++k) {
+    for (int k = 0; k < n + can_stay && st == LBM_OK && e == cudaSuccess; ++k) {
         // the shapes of the force model in use, timed with its step
         if (!step_shape_supported(L.precision, tx[k], ty[k])) continue;
         if (c->force_model == 1 && !pt_shape_supported(L.precision, tx[k], ty[k])) continue;
@@ -666,10 +723,12 @@ lbm_status lbm_autotune(lbm_ctx *c, int nsteps, int *best_tx, int *best_ty)
         refresh_maps(c);
         st = snapshot(c, snap, false);
         c->t = t0;
+        c->resident = k == n;
         for (int w = 0; w < 2 && e == cudaSuccess; ++w, ++c->t)
             e = launch_one_step(c, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-        for (int s = 0; s < nsteps && e == cudaSuccess; ++s, ++c->t)
+        int s = resident_steps(c, nsteps);
+        for (; s < nsteps && e == cudaSuccess; ++s, ++c->t)
             e = launch_one_step(c, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -683,6 +742,7 @@ lbm_status lbm_autotune(lbm_ctx *c, int nsteps, int *best_tx, int *best_ty)
     if (st == LBM_OK && e == cudaSuccess && best >= 0) {
         L.tx = tx[best];
         L.ty = ty[best];
+        c->resident = best == n;
         refresh_maps(c);
         st = snapshot(c, snap, false);
         c->t = t0;
@@ -715,7 +775,7 @@ lbm_status lbm_set_force_model(lbm_ctx *c, int model)
                     "LBM_F64 or LBM_F32");
     int tx, ty;
     pt_shape(c->L.precision, &tx, &ty);
-    lbm_status st = lbm_set_tile(c, tx, ty);
+    lbm_status st = change_tile(c, tx, ty);
     if (st != LBM_OK) return st;
     c->force_model = 1;
     return LBM_OK;
@@ -805,6 +865,7 @@ lbm_status lbm_step(lbm_ctx *c, int nsteps)
     if (!c->initialized) return fail(c, LBM_ERR_STATE, "lbm_init must come first");
     CUDA_TRY(c, cudaSetDevice(c->device));
     int left = nsteps;
+    left -= resident_steps(c, left);
     if (left > 0 && (c->t & 1)) {  // graphs start on an even step
         CUDA_TRY(c, launch_one_step(c, c->stream));
         ++c->t;

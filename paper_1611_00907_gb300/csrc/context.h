@@ -7,6 +7,7 @@
 
 #include "../../include/cplbm.h"
 #include "cplbm_internal.h"
+#include "resident.h"
 
 struct lbm_ctx {
     cplbm::Lattice L{};
@@ -33,6 +34,11 @@ struct lbm_ctx {
     cplbm::TmaMaps graph_maps{};
     int graph_force = -1;
     bool graph_failed = false;  // capture refused: direct launches only
+    // small lattices: blocks of steps with the state in shared memory
+    // (resident.cu); off once a tile shape has been chosen by the caller
+    cplbm::ResidentPlan plan;
+    bool resident = false;
+    unsigned xchg_tag = 1;      // next tag of L.xchg's words
     std::string err;
 };
 
@@ -41,6 +47,9 @@ namespace cplbm {
 // buffer of ctx_state_bytes(), or back (partial sums cleared).
 size_t ctx_state_bytes(const lbm_ctx *c);
 lbm_status ctx_snapshot(lbm_ctx *c, char *snap, bool save);
+// capi.cu: lbm_create; without the resident steps' exchange words when the
+// context belongs to a batch, which has its own.
+lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out);
 // capi.cu: rebuild the TMA maps after a tile-shape change.
 void ctx_refresh_maps(lbm_ctx *c);
 }  // namespace cplbm

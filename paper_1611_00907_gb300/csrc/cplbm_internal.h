@@ -95,6 +95,8 @@ struct Lattice {
     double mu_bottom, mu_top;
     int top_mode;
     int precision;
+    void *xchg;          // exchange words of the resident steps (resident.cu),
+                         // or null
     int *err;            // device flag: a bounded wait in a kernel gave up
     long long wait_cycles;  // SM clocks a tile waits for its staged data
                             // before it gives up (WAIT_CYCLES_DEFAULT)
@@ -103,7 +105,7 @@ struct Lattice {
 #ifdef CPLBM_CHECK_BOUNDS
     // bounds-checked build: bytes of pops, of each density buffer and of
     // each partial-sum class (set_bounds)
-    long long b_pops, b_rho, b_ring[R_COUNT];
+    long long b_pops, b_rho, b_ring[R_COUNT], b_xchg;
 #endif
 };
 

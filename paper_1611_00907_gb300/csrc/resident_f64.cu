@@ -1,0 +1,12 @@
+// Resident steps of one storage precision (SF64): see resident_impl.cuh.
+#include "resident_impl.cuh"
+
+namespace cplbm {
+
+cudaError_t launch_resident_f64(const ResidentArgs &a, bool batch, int grid, int threads,
+                              size_t smem, cudaStream_t s)
+{
+    return launch_resident_t<SF64>(a, batch, grid, threads, smem, s);
+}
+
+}  // namespace cplbm
