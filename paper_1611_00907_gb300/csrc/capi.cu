@@ -2,6 +2,7 @@
 // argument checks, EOS set-up and the host side of every call.
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -234,18 +235,6 @@ lbm_status ensure_tmp(lbm_ctx *c, size_t bytes)
     return LBM_OK;
 }
 
-// Queue the zeroing of both generations of partial sums.
-cudaError_t clear_rings(const Lattice &L, cudaStream_t s)
-{
-    const size_t rb = rho_bytes(L.precision);
-    for (int k = 0; k < 2; ++k)
-        for (int r = 0; r < R_COUNT; ++r) {
-            cudaError_t e = cudaMemsetAsync(L.ring[k][r], 0, ring_elems(L, r) * rb, s);
-            if (e != cudaSuccess) return e;
-        }
-    return cudaSuccess;
-}
-
 void free_all(lbm_ctx *c)
 {
     if (c->graph) cudaGraphExecDestroy(c->graph);
@@ -258,11 +247,9 @@ void free_all(lbm_ctx *c)
         dev_free(L.rho[k]);
         for (int r = 0; r < R_COUNT; ++r) dev_free(L.ring[k][r]);
     }
-    dev_free(c->d_red);
-    dev_free(c->d_bad);
+    dev_free(c->d_report);
     dev_free(c->d_prev);
     dev_free(c->d_tmp);
-    dev_free(c->d_err);
     dev_free(L.xchg);
 }
 
@@ -275,20 +262,26 @@ void refresh_maps(lbm_ctx *c)
     if (c->use_tma) build_tma_maps(c->L, &c->maps, msg, sizeof msg);
 }
 
-// Kernel error flags: a bounded wait inside a kernel gave up.
-lbm_status check_kernel_flags(lbm_ctx *c)
+lbm_status report_flags(lbm_ctx *c, int flags)
+{
+    if (!flags) return LBM_OK;
+    CUDA_TRY(c, cudaMemsetAsync(&c->d_report->err, 0, sizeof(int), c->stream));
+    if (flags & ERR_BOUNDS)
+        return fail(c, LBM_ERR_CUDA, "a kernel accessed memory outside its buffer "
+                    "(bounds-checked build; flags %d); the access was skipped", flags);
+    return fail(c, LBM_ERR_CUDA, "a step kernel's wait for its data timed out "
+                "(flags %d); the affected tiles were not updated", flags);
+}
+
+// Wait for the stream and report the kernels' error flags (a bounded wait
+// inside a kernel gave up); their copy is queued with the call's other ones.
+lbm_status finish(lbm_ctx *c)
 {
     int flags = 0;
-    CUDA_TRY(c, cudaMemcpy(&flags, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flags) {
-        CUDA_TRY(c, cudaMemset(c->d_err, 0, sizeof(int)));
-        if (flags & ERR_BOUNDS)
-            return fail(c, LBM_ERR_CUDA, "a kernel accessed memory outside its buffer "
-                        "(bounds-checked build; flags %d); the access was skipped", flags);
-        return fail(c, LBM_ERR_CUDA, "a step kernel's wait for its data timed out "
-                    "(flags %d); the affected tiles were not updated", flags);
-    }
-    return LBM_OK;
+    CUDA_TRY(c, cudaMemcpyAsync(&flags, &c->d_report->err, sizeof(int), cudaMemcpyDeviceToHost,
+                                c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    return report_flags(c, flags);
 }
 
 struct StateHeader {
@@ -469,10 +462,8 @@ lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
         alloc(&L.rho[k], (size_t)L.plane * rb);
         for (int r = 0; r < R_COUNT; ++r) alloc(&L.ring[k][r], ring_elems(L, r) * rb);
     }
-    alloc((void **)&c->d_red, 4 * sizeof(double));
-    alloc((void **)&c->d_bad, sizeof(int));
+    alloc((void **)&c->d_report, sizeof(Report));
     alloc((void **)&c->d_prev, (size_t)L.nx * L.ny * sizeof(double));
-    alloc((void **)&c->d_err, sizeof(int));
     const char *no_tma = getenv("CPLBM_NO_TMA");
     c->use_tma = !(no_tma && no_tma[0] == '1');
     if (alone && c->use_tma && st == LBM_OK && resident_plan(&L, 1, c->device, &c->plan)) {
@@ -485,14 +476,19 @@ lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
         if (c->resident && cudaMemsetAsync(L.xchg, 0, xchg_bytes(L), c->stream) != cudaSuccess)
             st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
     }
-    if (st == LBM_OK && cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess)
+    // the densities' row padding is loaded with the tiles and never written:
+    // zero, once
+    for (int k = 0; k < 2 && st == LBM_OK; ++k)
+        if (cudaMemsetAsync(L.rho[k], 0, (size_t)L.plane * rb, c->stream) != cudaSuccess)
+            st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
+    if (st == LBM_OK && cudaMemset(c->d_report, 0, sizeof(Report)) != cudaSuccess)
         st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
     if (st != LBM_OK) {
         free_all(c);
         delete c;
         return st;
     }
-    L.err = c->d_err;
+    L.err = &c->d_report->err;
     L.wait_cycles = WAIT_CYCLES_DEFAULT;
     refresh_maps(c);
     *out = c;
@@ -642,7 +638,7 @@ lbm_status change_tile(lbm_ctx *c, int tx, int ty)
         const int p = (int)(c->t & 1);
         CUDA_TRY(c, launch_gather_rho(L, p, L.rho[p ^ 1], c->stream));
         const size_t rb = rho_bytes(L.precision);
-        CUDA_TRY(c, clear_rings(L, c->stream));
+        CUDA_TRY(c, launch_clear_rings(L, c->stream));
         CUDA_TRY(c, cudaMemcpyAsync(L.rho[p], L.rho[p ^ 1], (size_t)L.plane * rb,
                                     cudaMemcpyDeviceToDevice, c->stream));
         CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -677,7 +673,7 @@ lbm_status snapshot(lbm_ctx *c, char *snap, bool save)
         CUDA_TRY(c, cudaMemcpyAsync(snap, L.pops, pb, cudaMemcpyDeviceToDevice,
                                     c->stream));
     } else {
-        CUDA_TRY(c, clear_rings(L, c->stream));
+        CUDA_TRY(c, launch_clear_rings(L, c->stream));
         CUDA_TRY(c, cudaMemcpyAsync(L.pops, snap, pb, cudaMemcpyDeviceToDevice,
                                     c->stream));
         CUDA_TRY(c, cudaMemcpyAsync(L.rho[p], snap + pb, rb,
@@ -832,19 +828,13 @@ lbm_status lbm_init(lbm_ctx *c, const double *rho, const double *ux,
             duy = t2;
         }
     }
-    const size_t rb = rho_bytes(L.precision);
-    for (int k = 0; k < 2; ++k)
-        CUDA_TRY(c, cudaMemsetAsync(L.rho[k], 0, (size_t)L.plane * rb, c->stream));
-    CUDA_TRY(c, clear_rings(L, c->stream));
-    CUDA_TRY(c, cudaMemsetAsync(c->d_bad, 0, sizeof(int), c->stream));
-    CUDA_TRY(c, launch_init(L, drho, dux, duy, c->d_bad, c->stream));
+    CUDA_TRY(c, launch_clear_rings(L, c->stream));
+    int *d_bad = &c->d_report->bad;
+    CUDA_TRY(c, cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
     // the reduction snapshot starts at the initial density
-    CUDA_TRY(c, cudaMemsetAsync(c->d_prev, 0, field, c->stream));
-    CUDA_TRY(c, launch_macro(L, 0, 0, c->d_prev, nullptr, nullptr, nullptr,
-                             nullptr, nullptr, nullptr, c->stream));
+    CUDA_TRY(c, launch_init(L, drho, dux, duy, c->d_prev, d_bad, c->stream));
     int bad = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(&bad, c->d_bad, sizeof(int), cudaMemcpyDeviceToHost,
-                                c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     c->t = 0;
     if (bad) {
@@ -896,8 +886,7 @@ lbm_status lbm_moments(lbm_ctx *c, double *rho, double *vx, double *vy,
     if (on_device) {
         CUDA_TRY(c, launch_macro(L, p, p, rho, vx, vy, mu, nullptr, nullptr,
                                  nullptr, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        return check_kernel_flags(c);
+        return finish(c);
     }
     lbm_status s = ensure_tmp(c, 4 * field);
     if (s != LBM_OK) return s;
@@ -910,12 +899,7 @@ lbm_status lbm_moments(lbm_ctx *c, double *rho, double *vx, double *vy,
         if (h[k])
             CUDA_TRY(c, cudaMemcpyAsync(h[k], d[k], field, cudaMemcpyDeviceToHost,
                                         c->stream));
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    {
-        lbm_status fs = check_kernel_flags(c);
-        if (fs != LBM_OK) return fs;
-    }
-    return LBM_OK;
+    return finish(c);
 }
 
 lbm_status lbm_get_populations(lbm_ctx *c, double *f, int on_device)
@@ -938,12 +922,7 @@ lbm_status lbm_get_populations(lbm_ctx *c, double *f, int on_device)
     CUDA_TRY(c, launch_populations(L, p, p, dst, c->stream));
     if (!on_device)
         CUDA_TRY(c, cudaMemcpyAsync(f, dst, bytes, cudaMemcpyDeviceToHost, c->stream));
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    {
-        lbm_status fs = check_kernel_flags(c);
-        if (fs != LBM_OK) return fs;
-    }
-    return LBM_OK;
+    return finish(c);
 }
 
 lbm_status lbm_reduce(lbm_ctx *c, double out[4])
@@ -954,22 +933,16 @@ lbm_status lbm_reduce(lbm_ctx *c, double out[4])
     if (!c->initialized) return fail(c, LBM_ERR_STATE, "lbm_init must come first");
     CUDA_TRY(c, cudaSetDevice(c->device));
     const int p = (int)(c->t & 1);
-    CUDA_TRY(c, cudaMemsetAsync(c->d_red, 0, 4 * sizeof(double), c->stream));
-    CUDA_TRY(c, cudaMemsetAsync(c->d_bad, 0, sizeof(int), c->stream));
-    CUDA_TRY(c, launch_macro(c->L, p, p, nullptr, nullptr, nullptr, nullptr,
-                             c->d_red, c->d_prev, c->d_bad, c->stream));
-    double h[4];
-    int bad = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(h, c->d_red, sizeof h, cudaMemcpyDeviceToHost,
-                                c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(&bad, c->d_bad, sizeof(int), cudaMemcpyDeviceToHost,
-                                c->stream));
+    Report *d = c->d_report, h;
+    CUDA_TRY(c, cudaMemsetAsync(d, 0, offsetof(Report, err), c->stream));
+    CUDA_TRY(c, launch_macro(c->L, p, p, nullptr, nullptr, nullptr, nullptr, d->red, c->d_prev,
+                             &d->bad, c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(&h, d, sizeof h, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    {
-        lbm_status fs = check_kernel_flags(c);
-        if (fs != LBM_OK) return fs;
-    }
-    for (int k = 0; k < 4; ++k) out[k] = h[k];
+    const lbm_status fs = report_flags(c, h.err);
+    if (fs != LBM_OK) return fs;
+    const int bad = h.bad;
+    for (int k = 0; k < 4; ++k) out[k] = h.red[k];
     if (bad)
         return fail(c, LBM_ERR_NUMERIC, "%d fluid node(s) with non-finite "
                     "density or momentum", bad);
@@ -1030,7 +1003,7 @@ lbm_status lbm_set_state(lbm_ctx *c, const void *buf, size_t bytes)
     const size_t pbytes = 8 * (size_t)L.plane * pop_bytes(L.precision);
     const size_t rbytes = (size_t)L.plane * rho_bytes(L.precision);
     const int p = (int)(h.t & 1);
-    CUDA_TRY(c, clear_rings(L, c->stream));
+    CUDA_TRY(c, launch_clear_rings(L, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(L.pops, in, pbytes, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(L.rho[p], in + pbytes, rbytes,
                                 cudaMemcpyHostToDevice, c->stream));

@@ -9,6 +9,13 @@
 #include "cplbm_internal.h"
 #include "resident.h"
 
+namespace cplbm {
+struct Report {
+    double red[4];
+    int bad, err;
+};
+}  // namespace cplbm
+
 struct lbm_ctx {
     cplbm::Lattice L{};
     int device = 0;
@@ -16,12 +23,12 @@ struct lbm_ctx {
     long long t = 0;
     bool eos_set = false, initialized = false;
     double T = 0, alpha = 1, Tc = 0, rhoc = 0;
-    double *d_red = nullptr;   // 4 reduction slots
-    int *d_bad = nullptr;      // error counter
+    // 4 reduction slots, then the error counter and the kernel error flags
+    // (Lattice::err): one copy reads them all
+    cplbm::Report *d_report = nullptr;
     double *d_prev = nullptr;  // density snapshot of lbm_reduce [ny][nx]
     double *d_tmp = nullptr;   // staging for host-side field transfers
     size_t tmp_bytes = 0;
-    int *d_err = nullptr;      // kernel error flags (Lattice::err)
     cplbm::TmaMaps maps{};            // tensor maps of the TMA interior path
     bool use_tma = true;
     int force_model = 0;       // 0 chemical potential (Eq. 12), 1 Eq. 5

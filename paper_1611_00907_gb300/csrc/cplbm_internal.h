@@ -14,8 +14,10 @@ enum Precision { P_F64 = 0, P_F32 = 1, P_F32_OFF = 2, P_F16_OFF = 3 };
 enum EosKind { EOS_VDW = 0, EOS_CS = 1, EOS_PR = 2, EOS_RKS = 3 };
 
 // Tile of the field kernels (moments, reductions): independent of the step.
+// The lower one for lattices too small to fill the GPU with the higher
+// (launch_macro).
 constexpr int FIELD_TILE_X = 64;
-constexpr int FIELD_TILE_Y = 16;
+constexpr int FIELD_TILE_Y = 16, FIELD_TILE_Y_SMALL = 4;
 // Threads of a step CTA.  The step's tile shape (tx x ty fluid nodes per
 // CTA) is a property of the lattice: it also fixes the grid on which the
 // step hands the next density over (see step.cu), so every kernel that reads
@@ -150,7 +152,7 @@ constexpr long long WAIT_CYCLES_DEFAULT = 2000000000LL;
 // Entries of partial-sum class c (R_L .. R_TR) of one generation: one
 // column per 32-wide tile column (L, R), one row per 16-high tile row
 // (B, T), one entry per such tile (corners); see ring_index.
-inline size_t ring_elems(const Lattice &L, int c)
+__host__ __device__ inline size_t ring_elems(const Lattice &L, int c)
 {
     const size_t ncx = ((size_t)L.nx + 31) / 32, ncy = ((size_t)L.nyf + 15) / 16;
     if (c == R_L || c == R_R) return ncx * L.nyf_pad;
@@ -318,10 +320,14 @@ cudaError_t launch_step_batch(const BatchList &w, int parity, int cur, int preci
 cudaError_t launch_fp64_math(const double *x, int n, double *lg, double *rc,
                              cudaStream_t s);
 // Equilibrium initial state from double fields [ny][nx] on the device:
-// fills pops (parity 0 order) and rho[0]/ring[0]; counts invalid densities
-// into *bad (device int, zeroed by the caller).
+// fills pops (parity 0 order) and rho[0], and prev (the snapshot of
+// launch_macro) at the fluid nodes; counts invalid densities into *bad
+// (device int, zeroed by the caller).  The partial sums are the caller's
+// (launch_clear_rings).
 cudaError_t launch_init(const Lattice &L, const double *rho, const double *ux,
-                        const double *uy, int *bad, cudaStream_t s);
+                        const double *uy, double *prev, int *bad, cudaStream_t s);
+// Zero both generations of partial sums.
+cudaError_t launch_clear_rings(const Lattice &L, cudaStream_t s);
 
 // Macroscopic fields of the state (any output may be NULL; [ny][nx]), and
 // optional FP64 reductions into red[0..3] (sum rho, sum rho vx, sum rho vy,

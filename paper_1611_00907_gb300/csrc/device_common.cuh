@@ -433,6 +433,14 @@ __device__ __forceinline__ long long aa_write_index(const Lattice &L,
     return pidx(L, i, row_wrap(L, rt), wrapi(x + ex(i), L.nx));
 }
 
+// Tile of a column or row: the compiled tile shapes are 32 or 64 wide and
+// 16, 24 or 32 high, so no division by a variable is needed.
+__device__ __forceinline__ int tile_x(const Lattice &L, int x) { return x >> (L.tx == 32 ? 5 : 6); }
+__device__ __forceinline__ int tile_y(const Lattice &L, int r)
+{
+    return L.ty == 24 ? r / 24 : r >> (L.ty == 16 ? 4 : 5);
+}
+
 // ---------------------------------------------------------------------------
 // Density of the current step at fluid node (x, r) in stored form (offset
 // precisions: rho - rho_ref): the tile-local sum in rho[cur] plus the
@@ -449,7 +457,7 @@ __device__ __forceinline__ typename S::real load_rho_stored(const Lattice &L,
     const rt *R = (const rt *)L.rho[cur];
     const rt *rp = R + fidx(L, r, x);
     real v = CPLBM_IN_RHO(L, cur, rp, 1) ? (real)*rp : real(0);
-    const int bx = x / L.tx, by = r / L.ty;
+    const int bx = tile_x(L, x), by = tile_y(L, r);
     const int lx = x - bx * L.tx, ly = r - by * L.ty;
     const int wx = min(L.tx, L.nx - bx * L.tx);
     const int wy = min(L.ty, L.nyf - by * L.ty);

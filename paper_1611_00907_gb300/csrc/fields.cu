@@ -3,22 +3,34 @@
 // the density gather used by checkpoints.
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 
 namespace cplbm {
 
 // ---------------------------------------------------------------------------
-// Initial state f_i = f_i^eq(rho, u) (Eq. 14) at every fluid node.
+// Initial state f_i = f_i^eq(rho, u) (Eq. 14) at every fluid node, evaluated
+// in FP64 whatever the storage and bound by the FP64 units: opposite
+// directions share the even part of Eq. 14 and the factors are applied once,
+// 35 FP64 instructions a node against 60 for the eight expressions written
+// out.  It leaves the snapshot of the reductions behind as well, which took a
+// pass of macro_kernel.  1500 x 1100 FP64: 203 + 320 -> 110 us.
+// A block takes 64 x 4 nodes.
 // ---------------------------------------------------------------------------
+constexpr int INIT_X = 64, INIT_Y = 4;
+
 template <class S>
-__global__ void init_kernel(const Lattice L, const double *rho_in,
-                            const double *ux_in, const double *uy_in, int *bad)
+__global__ void __launch_bounds__(INIT_X *INIT_Y)
+    init_kernel(const Lattice L, const double *rho_in, const double *ux_in,
+                const double *uy_in, double *prev, int *bad, int blocks_x)
 {
     using pop_t = typename S::pop_t;
     using rho_t = typename S::rho_t;
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (long long)L.nx * L.nyf) return;
-    const int x = (int)(n % L.nx), r = (int)(n / L.nx);
+    using real = typename S::real;
+    const int by = blockIdx.x / blocks_x, bx = blockIdx.x - by * blocks_x;
+    const int x = bx * INIT_X + threadIdx.x % INIT_X, r = by * INIT_Y + threadIdx.x / INIT_X;
+    if (x >= L.nx || r >= L.nyf) return;
     const long long g = (long long)(r + L.walls) * L.nx + x;  // lattice index
     const double rho = rho_in[g];
     const double ux = ux_in ? ux_in[g] : 0.0, uy = uy_in ? uy_in[g] : 0.0;
@@ -26,18 +38,39 @@ __global__ void init_kernel(const Lattice L, const double *rho_in,
     if (!(rho > 0.0 && rho < pole && isfinite(ux) && isfinite(uy)))
         atomicAdd(bad, 1);
     const double ref = S::offset ? L.rho_ref : 0.0;
-    const double usq = 1.5 * (ux * ux + uy * uy);
-    pop_t *A = (pop_t *)L.pops;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const double eu = ex(i) * ux + ey(i) * uy;
-        const double feq =
-            wgt<double>(i) * rho * (1.0 + 3.0 * eu + 4.5 * eu * eu - usq);
-        pop_t *p = A + pidx(L, i, r, x);
-        if (CPLBM_IN_POPS(L, p, 1)) st_real(p, (typename S::real)(feq - wgt<double>(i) * ref));
-    }
+    // f_i = w_i (rho (e +- 3 e_i.u) - ref), e = 1 + 4.5 (e_i.u)^2 - 1.5 u^2
+    const double c = 1.0 - 1.5 * (ux * ux + uy * uy);
+    const double sp = ux + uy, sm = ux - uy;
+    const double r1 = rho * (1.0 / 9.0), r5 = rho * (1.0 / 36.0);
+    pop_t *A = (pop_t *)L.pops + fidx(L, r, x);
+    auto pair = [&](int i, double w, double rw, double u) {
+        const double e = 4.5 * u * u + c, o = 3.0 * u;
+        pop_t *p = A + (i - 1) * L.plane, *q = A + (opp(i) - 1) * L.plane;
+        const double fp = S::offset ? rw * (e + o) - w * ref : rw * (e + o);
+        const double fq = S::offset ? rw * (e - o) - w * ref : rw * (e - o);
+        if (CPLBM_IN_POPS(L, p, 1)) st_real(p, (real)fp);
+        if (CPLBM_IN_POPS(L, q, 1)) st_real(q, (real)fq);
+    };
+    pair(1, 1.0 / 9.0, r1, ux);
+    pair(2, 1.0 / 9.0, r1, uy);
+    pair(5, 1.0 / 36.0, r5, sp);
+    pair(8, 1.0 / 36.0, r5, sm);
+    const rho_t stored = (rho_t)(rho - ref);
     rho_t *q = (rho_t *)L.rho[0] + fidx(L, r, x);
-    if (CPLBM_IN_RHO(L, 0, q, 1)) *q = (rho_t)(rho - ref);
+    if (CPLBM_IN_RHO(L, 0, q, 1)) *q = stored;
+    prev[g] = (double)((real)stored + (S::offset ? consts<real>(L).rho_ref : real(0)));
+}
+
+// Zero both generations of partial sums: block row k is generation k / 8,
+// class k % 8.  One launch where sixteen memsets stood.
+__global__ void clear_rings_kernel(const Lattice L, int words_per_entry)
+{
+    const int gen = blockIdx.y / R_COUNT, c = blockIdx.y % R_COUNT;
+    const long long n = (long long)ring_elems(L, c) * words_per_entry;
+    int *p = (int *)L.ring[gen][c];
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x)
+        p[i] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -51,14 +84,64 @@ __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v)
     atomicMax((unsigned long long *)addr, (unsigned long long)__double_as_longlong(v));
 }
 
+// FP64 values of FP32 results without the FP64 units, which do the type
+// conversions too (widen): subnormal values count as zero.
+__device__ __forceinline__ double to_f64(double v) { return v; }
+__device__ __forceinline__ double to_f64(float v)
+{
+    const unsigned mag = __float_as_uint(v) & 0x7FFFFFFFu;
+    if (mag >= 0x7F800000u) return (double)v;  // infinities, NaN
+    return widen(mag < 0x00800000u ? 0.0f : v);
+}
+// 1 / rho: IEEE division where rcp_nr has no answer (zero, infinite).
+__device__ __forceinline__ double inverse(double v)
+{
+    const unsigned e = (unsigned)__double2hiint(v) >> 20 & 0x7FFu;
+    return e > 1 && e < 0x7FDu ? rcp_nr(v) : 1.0 / v;
+}
+// v / 3 correctly rounded (normal v): the rounded product, corrected by its
+// exact remainder.
+__device__ __forceinline__ float third(float v)
+{
+    const float q = v * (1.0f / 3.0f);
+    return fmaf(fmaf(-3.0f, q, v), 1.0f / 3.0f, q);
+}
+// rho v = j + F / 2 of a node (momentum, force of Eq. 12 from the 12 grad).
+__device__ __forceinline__ void half_force(const Consts<float> &, const float *f, float rho,
+                                           float grx, float gry, float gmx, float gmy,
+                                           double &px, double &py)
+{
+    const float c = 1.0f / 12.0f;
+    const float Fx = -rho * (gmx * c) + third(grx * c), Fy = -rho * (gmy * c) + third(gry * c);
+    const float jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
+    const float jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
+    px = to_f64(jx) + 0.5 * to_f64(Fx);
+    py = to_f64(jy) + 0.5 * to_f64(Fy);
+}
+__device__ __forceinline__ void half_force(const Consts<double> &, const double *f, double rho,
+                                           double grx, double gry, double gmx, double gmy,
+                                           double &px, double &py)
+{
+    double jx, jy;
+    momentum(f, jx, jy);
+    const double r = rho * (-1.0 / 24.0);
+    px = (1.0 / 72.0) * grx + (r * gmx + jx);
+    py = (1.0 / 72.0) * gry + (r * gmy + jy);
+}
+
+// Bound by the FP64 units, in FP64 (67 FP64 instructions a node) and, with
+// velocities or reductions, in FP32 too (the division and the sums are FP64
+// in every storage).  1500 x 1100 FP64: 367 -> 190 us for the four fields.
 template <class S, int TX, int TY>
-__global__ void macro_kernel(const Lattice L, int parity, int cur,
-                             double *o_rho, double *o_vx, double *o_vy,
-                             double *o_mu, double *red, double *prev, int *bad)
+__global__ void __launch_bounds__(256)
+    macro_kernel(const Lattice L, int parity, int cur, double *o_rho, double *o_vx,
+                 double *o_vy, double *o_mu, double *red, double *prev, int *bad)
 {
     using real = typename S::real;
     using pop_t = typename S::pop_t;
     constexpr int WR = TX + 4, WM = TX + 2;
+    constexpr int PER = TX * TY / 256;   // rows of a thread, one above the other
+    static_assert(PER * 256 == TX * TY, "whole columns of rows");
     extern __shared__ unsigned char smem_raw[];
     real *s_rho = reinterpret_cast<real *>(smem_raw);
     real *s_mu = s_rho + (TY + 4) * WR;
@@ -73,49 +156,61 @@ __global__ void macro_kernel(const Lattice L, int parity, int cur,
     mu_tile<S, TX, TY>(L, X0, Y0, s_rho, s_mu);
     __syncthreads();
 
-    const real rho_ref = S::offset ? consts<real>(L).rho_ref : real(0);
+    const Consts<real> &K = consts<real>(L);
+    const real rho_ref = S::offset ? K.rho_ref : real(0);
     const pop_t *A = (const pop_t *)L.pops;
+    const bool flow = o_vx || o_vy || red;   // otherwise no population is needed
     double acc_m = 0.0, acc_x = 0.0, acc_y = 0.0, acc_d = 0.0;
     // s_rho holds the stored form; rho_ref makes it absolute
     int nbad = 0;
-    for (int n = threadIdx.x; n < TX * TY; n += blockDim.x) {
-        const int lx = n % TX, ly = n / TX;
-        if (lx >= wx || ly >= wy) continue;
-        const int x = X0 + lx, r = Y0 + ly;
-        const int cr = (ly + 2) * WR + lx + 2, cm = (ly + 1) * WM + lx + 1;
-        real f[9];
+    const int lx = threadIdx.x % TX, ly0 = threadIdx.x / TX * PER;
+    const int cr0 = (ly0 + 1) * WR + lx + 2, cm0 = ly0 * WM + lx + 1;
+    Row<real> rd = row_of(s_rho, cr0), rm = row_of(s_rho, cr0 + WR);
+    Row<real> md = row_of(s_mu, cm0), mm = row_of(s_mu, cm0 + WM);
 #pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            const pop_t *p = A + aa_read_index(L, parity, i, r, x);
-            f[i] = CPLBM_IN_POPS(L, p, 1) ? ld_real(p) : real(0);
-        }
-        const real rho = s_rho[cr] + rho_ref;
-        real gmx, gmy, grx, gry;
-        grad9<real, WM>(s_mu, cm, gmx, gmy);
-        grad9<real, WR>(s_rho, cr, grx, gry);
-        const real Fx = -rho * gmx + grx / real(3);
-        const real Fy = -rho * gmy + gry / real(3);
-        const real jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
-        const real jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
-        const double px = (double)jx + 0.5 * (double)Fx;  // rho v
-        const double py = (double)jy + 0.5 * (double)Fy;
-        const long long g = (long long)(r + L.walls) * L.nx + x;
-        if (o_rho) o_rho[g] = (double)rho;
-        if (o_vx) o_vx[g] = px / (double)rho;
-        if (o_vy) o_vy[g] = py / (double)rho;
-        if (o_mu) o_mu[g] = (double)s_mu[cm];
-        if (red) {
-            acc_m += (double)rho;
-            acc_x += px;
-            acc_y += py;
-            if (!(isfinite((double)rho) && isfinite(px) && isfinite(py)))
-                ++nbad;
-            if (prev) {
-                const double d = fabs((double)rho - prev[g]);
-                acc_d = fmax(acc_d, isfinite(d) ? d : 0.0);
-                prev[g] = (double)rho;
+    for (int k = 0; k < PER; ++k) {
+        const int ly = ly0 + k;
+        const Row<real> ru = row_of(s_rho, cr0 + (k + 2) * WR);
+        const Row<real> mu = row_of(s_mu, cm0 + (k + 2) * WM);
+        if (lx < wx && ly < wy) {
+            const int x = X0 + lx, r = Y0 + ly;
+            const long long g = (long long)(r + L.walls) * L.nx + x;
+            const real rho = rm.c + rho_ref;
+            const double rho64 = to_f64(rho);
+            if (o_rho) o_rho[g] = rho64;
+            if (o_mu) o_mu[g] = to_f64(mm.c);
+            if (flow) {
+                real f[9];
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    const pop_t *p = A + aa_read_index(L, parity, i, r, x);
+                    f[i] = CPLBM_IN_POPS(L, p, 1) ? ld_real(p) : real(0);
+                }
+                real grx, gry, gmx, gmy;
+                grad12(ru, rm, rd, grx, gry);
+                grad12(mu, mm, md, gmx, gmy);
+                double px, py;  // rho v
+                half_force(K, f, rho, grx, gry, gmx, gmy, px, py);
+                const double ir = inverse(rho64);
+                if (o_vx) o_vx[g] = px * ir;
+                if (o_vy) o_vy[g] = py * ir;
+                if (red) {
+                    acc_m += rho64;
+                    acc_x += px;
+                    acc_y += py;
+                    if (!(isfinite(rho64) && isfinite(px) && isfinite(py))) ++nbad;
+                    if (prev) {
+                        const double d = fabs(rho64 - prev[g]);
+                        acc_d = fmax(acc_d, isfinite(d) ? d : 0.0);
+                        prev[g] = rho64;
+                    }
+                }
             }
         }
+        rd = rm;
+        rm = ru;
+        md = mm;
+        mm = mu;
     }
     // Solid rows: rho by Eq. 28 and the wall mu from the shared tiles.
     if (L.walls && (o_rho || o_mu || o_vx || o_vy)) {
@@ -214,28 +309,42 @@ static inline unsigned blocks_for(long long n, int t)
 
 template <class S>
 static cudaError_t launch_init_t(const Lattice &L, const double *rho,
-                                 const double *ux, const double *uy, int *bad,
-                                 cudaStream_t s)
+                                 const double *ux, const double *uy, double *prev,
+                                 int *bad, cudaStream_t s)
 {
-    const long long n = (long long)L.nx * L.nyf;
-    init_kernel<S><<<blocks_for(n, 256), 256, 0, s>>>(L, rho, ux, uy, bad);
+    const int bx = (L.nx + INIT_X - 1) / INIT_X, by = (L.nyf + INIT_Y - 1) / INIT_Y;
+    init_kernel<S><<<(unsigned)bx * (unsigned)by, INIT_X * INIT_Y, 0, s>>>(L, rho, ux, uy, prev,
+                                                                          bad, bx);
     return cudaGetLastError();
 }
 
-template <class S>
-static cudaError_t launch_macro_t(const Lattice &L, int parity, int cur,
-                                  double *rho, double *vx, double *vy,
-                                  double *mu, double *red, double *prev,
-                                  int *bad, cudaStream_t s)
+template <class S, int TY>
+static cudaError_t launch_macro_ty(const Lattice &L, int parity, int cur, double *rho,
+                                   double *vx, double *vy, double *mu, double *red,
+                                   double *prev, int *bad, cudaStream_t s)
 {
     using real = typename S::real;
-    constexpr int TX = FIELD_TILE_X, TY = FIELD_TILE_Y;
-    const size_t smem =
-        sizeof(real) * ((TY + 4) * (TX + 4) + (TY + 2) * (TX + 2));
+    constexpr int TX = FIELD_TILE_X;
+    const size_t smem = sizeof(real) * ((TY + 4) * (TX + 4) + (TY + 2) * (TX + 2));
     dim3 grid((L.nx + TX - 1) / TX, (L.nyf + TY - 1) / TY);
-    macro_kernel<S, TX, TY><<<grid, 256, smem, s>>>(L, parity, cur, rho, vx,
-                                                     vy, mu, red, prev, bad);
+    macro_kernel<S, TX, TY><<<grid, 256, smem, s>>>(L, parity, cur, rho, vx, vy, mu, red, prev,
+                                                    bad);
     return cudaGetLastError();
+}
+
+// Tiles of 64 x 16, or of 64 x 4 (a quarter of the work per block, half of
+// it halo) while 64 x 16 would leave SMs without a block.
+template <class S>
+static cudaError_t launch_macro_t(const Lattice &L, int parity, int cur, double *rho, double *vx,
+                                  double *vy, double *mu, double *red, double *prev, int *bad,
+                                  cudaStream_t s)
+{
+    const long long tiles = (long long)((L.nx + FIELD_TILE_X - 1) / FIELD_TILE_X) *
+                            ((L.nyf + FIELD_TILE_Y - 1) / FIELD_TILE_Y);
+    return tiles < 152 ? launch_macro_ty<S, FIELD_TILE_Y_SMALL>(L, parity, cur, rho, vx, vy, mu,
+                                                                red, prev, bad, s)
+                       : launch_macro_ty<S, FIELD_TILE_Y>(L, parity, cur, rho, vx, vy, mu, red,
+                                                          prev, bad, s);
 }
 
 template <class S>
@@ -266,9 +375,18 @@ static cudaError_t launch_gather_t(const Lattice &L, int cur, void *dst,
     return cudaErrorInvalidValue;
 
 cudaError_t launch_init(const Lattice &L, const double *rho, const double *ux,
-                        const double *uy, int *bad, cudaStream_t s)
+                        const double *uy, double *prev, int *bad, cudaStream_t s)
 {
-    CPLBM_DISPATCH(L.precision, launch_init_t<S>(L, rho, ux, uy, bad, s))
+    CPLBM_DISPATCH(L.precision, launch_init_t<S>(L, rho, ux, uy, prev, bad, s))
+}
+
+cudaError_t launch_clear_rings(const Lattice &L, cudaStream_t s)
+{
+    const int words = (int)rho_bytes(L.precision) / 4;
+    const size_t most = std::max(ring_elems(L, R_L), ring_elems(L, R_B)) * words;
+    const unsigned blocks = (unsigned)std::min<size_t>((most + 255) / 256, 64);
+    clear_rings_kernel<<<dim3(blocks, 2 * R_COUNT), 256, 0, s>>>(L, words);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_macro(const Lattice &L, int parity, int cur, double *rho,

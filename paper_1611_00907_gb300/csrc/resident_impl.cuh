@@ -185,7 +185,7 @@ template <class rt>
 __device__ __forceinline__ void store_rho_whole(const Lattice &L, int gen, int r, int x, rt v)
 {
     put_rho(L, gen, (rt *)L.rho[gen], fidx(L, r, x), v);
-    const int bx = x / L.tx, by = r / L.ty;
+    const int bx = tile_x(L, x), by = tile_y(L, r);
     const int lx = x - bx * L.tx, ly = r - by * L.ty;
     const bool left = lx == 0, right = lx == min(L.tx, L.nx - bx * L.tx) - 1;
     const bool below = ly == 0 && !(L.walls && r == 0);
