@@ -4,16 +4,27 @@
 //
 // Network: 16 inputs (the caller's features, zero-padded) -> 3 hidden layers
 // of 128 tanh units -> 16 outputs (zero-padded; linear).  Each layer keeps
-// FP32 master weights (Adam state beside them) and two BF16 copies: W^T
-// [n][k] for the forward product and W [k][n] for back-propagation.
+// FP32 master weights (Adam state beside them) and two BF16 copies, for the
+// forward product and for back-propagation.
 //
-// One CTA of 4 warps handles 64 samples; each warp owns 16 samples (the M
-// dimension of the MMA).  Training is full-batch gradient descent: a CTA
-// back-propagates its samples and adds its weight gradients into FP32
-// accumulators with atomics; the Adam kernel then updates every weight.
+// Everything here is latency: the network is 37 000 parameters, an iteration
+// of 1024 samples 0.2 GFLOP.  A CTA takes 16 samples at a time, so that a
+// thousand samples are 64 CTAs, and its eight warps split each layer's
+// outputs; a warp's weights go straight from L2 to registers, in the order
+// the MMA wants them (fragment order, written by the Adam kernel), all loads
+// ahead of the first product.  Activations and deltas stay in padded shared
+// memory and reach the MMA by ldmatrix, transposed for the weight gradients.
+// Training is full-batch gradient descent: a CTA back-propagates its samples
+// and adds its weight gradients into FP32 accumulators (pairs per reduction);
+// the Adam kernel then updates every weight.  1024 samples: 161 us an
+// iteration with 64 samples and four warps per CTA, weights and activations
+// read from unpadded shared memory; now 14 us, a chain of eight products with
+// their barriers, the gradient's reductions and the Adam pass, whose launches
+// overlap by programmatic dependent launch.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <new>
@@ -26,7 +37,8 @@
 namespace cplbm_mlp {
 
 constexpr int DIN = 16, H = 128, DOUT = 16, NL = 4;
-constexpr int SAMPLES = 64, WARPS = 4, THREADS = 32 * WARPS;
+constexpr int SAMPLES = 16, WARPS = 8, THREADS = 32 * WARPS;
+constexpr int MAX_CTAS = 152;   // one per SM; more samples take several rounds
 __host__ __device__ constexpr int layer_k(int l) { return l == 0 ? DIN : H; }
 __host__ __device__ constexpr int layer_n(int l) { return l == NL - 1 ? DOUT : H; }
 
@@ -44,231 +56,359 @@ __host__ __device__ constexpr int b_off(int l)
 constexpr int NPARAM = b_off(NL);
 
 struct Params {
-    const __nv_bfloat16 *wt;  // W^T [n][k] per layer, BF16, at w_off(l)
-    const __nv_bfloat16 *w;   // W [k][n] per layer, BF16, at w_off(l)
+    const __nv_bfloat16 *wt;  // forward weights in fragment order, BF16, at w_off(l)
+    const __nv_bfloat16 *w;   // back-propagation weights likewise
     const float *p;           // FP32 masters (biases read from here)
 };
 
+// Fragment order of a B operand of mma.m16n8k16 (PTX ISA; lane = 4 g + t):
+// output column `col`, contraction index `kk` of KK.  A lane's four values of
+// a 16-deep step lie together, two steps side by side where there are two,
+// so that a lane's share of a column tile is a run of 16-byte words.
+__host__ __device__ constexpr int frag_pos(int col, int kk, int KK)
+{
+    const int j = col / 8, g = col % 8, step = kk / 16, r = kk % 16;
+    const int lane = 4 * g + (r % 8) / 2, e = (r & 1) + (r >= 8 ? 2 : 0);
+    return KK == 16 ? (j * 32 + lane) * 4 + e
+                    : ((j * (KK / 32) + step / 2) * 32 + lane) * 8 + (step & 1) * 4 + e;
+}
+
 // ---------------------------------------------------------------------------
-// Warp-level GEMM: acc[16 x N] += A[16 x K] * B[K x N].  A row-major in
-// shared memory (lda elements per row), B given as Bt[n][k] (ldb per n).
-// Fragment layouts of mma.m16n8k16 (PTX ISA): lane = 4 g + t.
+// mma.m16n8k16 BF16 -> FP32 and its fragments.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned ld_pair(const __nv_bfloat16 *p)
+struct FragA {
+    unsigned r[4];
+};
+__device__ __forceinline__ void mma(float (&acc)[4], const FragA &a, unsigned b0, unsigned b1)
 {
-    return *reinterpret_cast<const unsigned *>(p);
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
+        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
+        : "r"(a.r[0]), "r"(a.r[1]), "r"(a.r[2]), "r"(a.r[3]), "r"(b0), "r"(b1));
+}
+template <bool TRANS>
+__device__ __forceinline__ FragA ldmatrix4(const __nv_bfloat16 *p)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(p);
+    FragA f;
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                     : "=r"(f.r[0]), "=r"(f.r[1]), "=r"(f.r[2]), "=r"(f.r[3]) : "r"(s) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                     : "=r"(f.r[0]), "=r"(f.r[1]), "=r"(f.r[2]), "=r"(f.r[3]) : "r"(s) : "memory");
+    return f;
+}
+// A operand from row-major [16][...] at column k0 (row stride LD).
+template <int LD>
+__device__ __forceinline__ FragA frag_a(const __nv_bfloat16 *m, int k0)
+{
+    const int lane = threadIdx.x & 31;
+    return ldmatrix4<false>(m + (lane & 15) * LD + k0 + (lane >> 4) * 8);
+}
+// A operand of the transpose: rows are columns k0 .. k0 + 15 of m, the
+// contraction runs over m's 16 rows.
+template <int LD>
+__device__ __forceinline__ FragA frag_at(const __nv_bfloat16 *m, int k0)
+{
+    const int lane = threadIdx.x & 31;
+    return ldmatrix4<true>(m + ((lane & 7) + (lane >> 4) * 8) * LD + k0 + ((lane >> 3) & 1) * 8);
+}
+// B operands of two column tiles n0, n0 + 8 of m [16][...], contraction over
+// its rows: {b0, b1} of the first tile, then of the second.
+template <int LD>
+__device__ __forceinline__ FragA frag_b2(const __nv_bfloat16 *m, int n0)
+{
+    const int lane = threadIdx.x & 31;
+    return ldmatrix4<true>(m + ((lane & 7) + ((lane >> 3) & 1) * 8) * LD + n0 + (lane >> 4) * 8);
 }
 
-template <int K, int N>
-__device__ __forceinline__ void warp_gemm(const __nv_bfloat16 *A, int lda,
-                                          const __nv_bfloat16 *Bt, int ldb,
-                                          float (&acc)[N / 8][4])
-{
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        const unsigned a0 = ld_pair(A + g * lda + k0 + 2 * t);
-        const unsigned a1 = ld_pair(A + (g + 8) * lda + k0 + 2 * t);
-        const unsigned a2 = ld_pair(A + g * lda + k0 + 8 + 2 * t);
-        const unsigned a3 = ld_pair(A + (g + 8) * lda + k0 + 8 + 2 * t);
-#pragma unroll
-        for (int j = 0; j < N / 8; ++j) {
-            const __nv_bfloat16 *bp = Bt + (j * 8 + g) * ldb + k0 + 2 * t;
-            const unsigned b0 = ld_pair(bp), b1 = ld_pair(bp + 8);
-            asm volatile(
-                "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-                "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-                "{%0, %1, %2, %3};\n"
-                : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
-                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-        }
-    }
-}
+// Rows of 16 and 128 values, padded so that the eight rows an ldmatrix reads
+// lie in different banks.
+constexpr int LD16 = 24, LD128 = 136;
 
-// Element (row, col) held by accumulator slot q of n-tile j.
-__device__ __forceinline__ void acc_pos(int j, int q, int &row, int &col)
-{
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    row = g + (q >= 2 ? 8 : 0);
-    col = j * 8 + 2 * t + (q & 1);
-}
-
-// Shared memory of one CTA.
 struct Smem {
-    __nv_bfloat16 wt[H * H];                // current layer's Bt operand
-    __nv_bfloat16 act[NL][SAMPLES * H];     // inputs of layer l, [s][k]
-    __nv_bfloat16 actT[NL][H * SAMPLES];    // the same, [k][s]
-    __nv_bfloat16 dlt[SAMPLES * H];         // delta of the current layer [s][n]
-    __nv_bfloat16 dltT[H * SAMPLES];        // [n][s]
+    __nv_bfloat16 in[SAMPLES * LD16];           // input of layer 0, [s][k]
+    __nv_bfloat16 act[NL - 1][SAMPLES * LD128]; // inputs of layers 1 .. 3
+    __nv_bfloat16 dout[SAMPLES * LD16];         // output delta [s][n]
+    __nv_bfloat16 dlt[2][SAMPLES * LD128];      // deltas of the hidden layers
     float out[SAMPLES * DOUT];
 };
 
-__device__ void load_bt(__nv_bfloat16 *dst, const __nv_bfloat16 *src, int n)
+// A warp's weights: its two column tiles of each 128-column layer (layer 3's
+// forward product has two tiles in all: one each for the first two warps).
+struct Weights {
+    uint2 in[2];          // layer 0 forward (16 deep)
+    uint4 f1[2][4], f2[2][4], f3[4];
+    uint2 b3[2];          // back-propagation through layer 3 (16 deep)
+    uint4 b2[2][4], b1[2][4];
+};
+__device__ __forceinline__ uint4 load16(const __nv_bfloat16 *w, int tile, int k2)
 {
-    for (int q = threadIdx.x; q < n; q += THREADS) dst[q] = src[q];
+    return reinterpret_cast<const uint4 *>(w)[(tile * 4 + k2) * 32 + (threadIdx.x & 31)];
 }
-
-// Forward pass of the CTA's 64 samples; stores every layer's input
-// (row-major and transposed) and the FP32 outputs.
-__device__ void forward(const Params &P, Smem &S)
+template <bool BACK>
+__device__ __forceinline__ void load_weights(const Params &P, Weights &W)
 {
-    const int warp = threadIdx.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int l = 0; l < NL; ++l) {
-        constexpr int dummy = 0;
-        (void)dummy;
-        const int K = layer_k(l), N = layer_n(l);
-        load_bt(S.wt, P.wt + w_off(l), K * N);
-        __syncthreads();
-        const __nv_bfloat16 *A = S.act[l] + warp * 16 * K;
-        if (N == H) {
-            float acc[H / 8][4] = {};
-            if (K == DIN) warp_gemm<DIN, H>(A, K, S.wt, K, acc);
-            else warp_gemm<H, H>(A, K, S.wt, K, acc);
+    for (int q = 0; q < 2; ++q) {
+        const int j = 2 * warp + q;
+        W.in[q] = reinterpret_cast<const uint2 *>(P.wt + w_off(0))[j * 32 + lane];
 #pragma unroll
-            for (int j = 0; j < H / 8; ++j)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    int r, c;
-                    acc_pos(j, q, r, c);
-                    const float v = tanhf(acc[j][q] + P.p[b_off(l) + c]);
-                    const int s = warp * 16 + r;
-                    const __nv_bfloat16 bv = __float2bfloat16(v);
-                    S.act[l + 1][s * H + c] = bv;
-                    S.actT[l + 1][c * SAMPLES + s] = bv;
-                }
-        } else {
-            float acc[DOUT / 8][4] = {};
-            warp_gemm<H, DOUT>(A, K, S.wt, K, acc);
-#pragma unroll
-            for (int j = 0; j < DOUT / 8; ++j)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    int r, c;
-                    acc_pos(j, q, r, c);
-                    S.out[(warp * 16 + r) * DOUT + c] = acc[j][q] + P.p[b_off(l) + c];
-                }
+        for (int k = 0; k < 4; ++k) {
+            W.f1[q][k] = load16(P.wt + w_off(1), j, k);
+            W.f2[q][k] = load16(P.wt + w_off(2), j, k);
         }
-        __syncthreads();
+    }
+    if (warp < 2)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) W.f3[k] = load16(P.wt + w_off(3), warp, k);
+    if (BACK) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int j = 2 * warp + q;
+            W.b3[q] = reinterpret_cast<const uint2 *>(P.w + w_off(3))[j * 32 + lane];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                W.b2[q][k] = load16(P.w + w_off(2), j, k);
+                W.b1[q][k] = load16(P.w + w_off(1), j, k);
+            }
+        }
     }
 }
 
-__device__ void load_inputs(Smem &S, const float *X, int nin, int B, int s0)
+// acc[q] = (16 x 128 at m) * (the warp's column tile q), contraction in
+// ascending order.
+template <int NT>
+__device__ __forceinline__ void product(const __nv_bfloat16 *m, const uint4 (*w)[4],
+                                        float (&acc)[NT][4])
 {
-    for (int q = threadIdx.x; q < SAMPLES * DIN; q += THREADS) {
-        const int s = q / DIN, k = q % DIN, gs = s0 + s;
-        const float v = (gs < B && k < nin) ? X[(long long)gs * nin + k] : 0.f;
-        const __nv_bfloat16 bv = __float2bfloat16(v);
-        S.act[0][s * DIN + k] = bv;
-        S.actT[0][k * SAMPLES + s] = bv;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const FragA a0 = frag_a<LD128>(m, 32 * k), a1 = frag_a<LD128>(m, 32 * k + 16);
+#pragma unroll
+        for (int q = 0; q < NT; ++q) mma(acc[q], a0, w[q][k].x, w[q][k].y);
+#pragma unroll
+        for (int q = 0; q < NT; ++q) mma(acc[q], a1, w[q][k].z, w[q][k].w);
+    }
+}
+// Two adjacent values as a BF16 pair at row r, column c of m.
+__device__ __forceinline__ void put2(__nv_bfloat16 *m, int r, int c, float x, float y)
+{
+    *reinterpret_cast<__nv_bfloat162 *>(m + r * LD128 + c) = __floats2bfloat162_rn(x, y);
+}
+__device__ __forceinline__ float2 get2(const __nv_bfloat16 *m, int r, int c)
+{
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(m + r * LD128 + c));
+}
+// tanh(acc + bias) of the warp's tiles into m.
+__device__ __forceinline__ void activate(const float (&acc)[2][4], const float2 (&bias)[2],
+                                         __nv_bfloat16 *m)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int c = ((threadIdx.x >> 5) * 2 + q) * 8 + 2 * t;
+        put2(m, g, c, tanhf(acc[q][0] + bias[q].x), tanhf(acc[q][1] + bias[q].y));
+        put2(m, g + 8, c, tanhf(acc[q][2] + bias[q].x), tanhf(acc[q][3] + bias[q].y));
+    }
+}
+struct Biases {
+    float2 h[NL - 1][2], out;
+};
+__device__ __forceinline__ void load_biases(const Params &P, Biases &B)
+{
+    const int warp = threadIdx.x >> 5, t = threadIdx.x & 3;
+#pragma unroll
+    for (int l = 0; l < NL - 1; ++l)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            B.h[l][q] = *reinterpret_cast<const float2 *>(P.p + b_off(l) + (2 * warp + q) * 8 + 2 * t);
+    if (warp < 2) B.out = *reinterpret_cast<const float2 *>(P.p + b_off(NL - 1) + warp * 8 + 2 * t);
+}
+
+// Forward pass of the CTA's 16 samples from s0 on: every layer's input and
+// the FP32 outputs in S.  Ends with a barrier.
+__device__ __forceinline__ void forward(const Weights &W, const Biases &Bs, Smem &S,
+                                        const float *X, int nin, int B, int s0)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    {
+        const int s = threadIdx.x / DIN, k = threadIdx.x % DIN;
+        const float v = s0 + s < B && k < nin ? X[(long long)(s0 + s) * nin + k] : 0.f;
+        S.in[s * LD16 + k] = __float2bfloat16(v);
+    }
+    __syncthreads();
+    {
+        float acc[2][4] = {};
+        const FragA a = frag_a<LD16>(S.in, 0);
+        mma(acc[0], a, W.in[0].x, W.in[0].y);
+        mma(acc[1], a, W.in[1].x, W.in[1].y);
+        activate(acc, Bs.h[0], S.act[0]);
+    }
+    __syncthreads();
+    {
+        float acc[2][4] = {};
+        product<2>(S.act[0], W.f1, acc);
+        activate(acc, Bs.h[1], S.act[1]);
+    }
+    __syncthreads();
+    {
+        float acc[2][4] = {};
+        product<2>(S.act[1], W.f2, acc);
+        activate(acc, Bs.h[2], S.act[2]);
+    }
+    __syncthreads();
+    if (warp < 2) {
+        float acc[1][4] = {};
+        product<1>(S.act[2], &W.f3, acc);
+        const int g = lane >> 2, c = warp * 8 + 2 * (lane & 3);
+        float *o = S.out + g * DOUT + c;
+        o[0] = acc[0][0] + Bs.out.x;
+        o[1] = acc[0][1] + Bs.out.y;
+        o[8 * DOUT] = acc[0][2] + Bs.out.x;
+        o[8 * DOUT + 1] = acc[0][3] + Bs.out.y;
     }
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(THREADS)
+// Programmatic dependent launch: a kernel lets its successor start while it
+// runs, and touches memory only once its predecessor has ended.
+__device__ __forceinline__ void after_predecessor()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
     mlp_infer_kernel(Params P, const float *X, int nin, float *Y, int nout, int B)
 {
-    extern __shared__ __align__(16) unsigned char raw[];
-    Smem &S = *reinterpret_cast<Smem *>(raw);
-    const int s0 = blockIdx.x * SAMPLES;
-    load_inputs(S, X, nin, B, s0);
-    forward(P, S);
-    for (int q = threadIdx.x; q < SAMPLES * nout; q += THREADS) {
-        const int s = q / nout, c = q % nout;
-        if (s0 + s < B) Y[(long long)(s0 + s) * nout + c] = S.out[s * DOUT + c];
+    __shared__ __align__(16) Smem S;
+    Weights W;
+    Biases Bs;
+    load_weights<false>(P, W);
+    load_biases(P, Bs);
+    for (int s0 = blockIdx.x * SAMPLES; s0 < B; s0 += gridDim.x * SAMPLES) {
+        forward(W, Bs, S, X, nin, B, s0);
+        const int s = threadIdx.x / DOUT, c = threadIdx.x % DOUT;
+        if (s0 + s < B && c < nout) Y[(long long)(s0 + s) * nout + c] = S.out[threadIdx.x];
+        __syncthreads();
     }
+}
+
+__device__ __forceinline__ void add2(float *p, float x, float y)
+{
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(x), "f"(y)
+                 : "memory");
+}
+// Weight gradient dW[k][n] += sum_s a[s][k] d[s][n] of the rows k0 .. k0 + 15
+// and the column tiles n0 .. n0 + 8 (NT - 1) of a layer with N columns.
+template <int LDA, int LDD, int N, int NT>
+__device__ __forceinline__ void weight_grad(const __nv_bfloat16 *a, const __nv_bfloat16 *d,
+                                            int k0, int n0, float *grad)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const FragA at = frag_at<LDA>(a, k0);
+    float *o = grad + (k0 + g) * N + n0 + 2 * t;
+#pragma unroll
+    for (int q = 0; q < NT; q += 2) {
+        const FragA b = frag_b2<LDD>(d, n0 + 8 * q);
+        float x[4] = {}, y[4] = {};
+        mma(x, at, b.r[0], b.r[1]);
+        mma(y, at, b.r[2], b.r[3]);
+        add2(o + 8 * q, x[0], x[1]);
+        add2(o + 8 * q + 8 * N, x[2], x[3]);
+        add2(o + 8 * q + 8, y[0], y[1]);
+        add2(o + 8 * q + 8 + 8 * N, y[2], y[3]);
+    }
+}
+// Delta of a hidden layer from acc = (delta above) W^T: acc (1 - a^2), a the
+// layer's output; samples beyond B have a zero delta above.
+__device__ __forceinline__ void hidden_delta(const float (&acc)[2][4], const __nv_bfloat16 *a,
+                                             __nv_bfloat16 *d)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int c = ((threadIdx.x >> 5) * 2 + q) * 8 + 2 * t;
+        const float2 u = get2(a, g, c), v = get2(a, g + 8, c);
+        put2(d, g, c, acc[q][0] * (1.f - u.x * u.x), acc[q][1] * (1.f - u.y * u.y));
+        put2(d, g + 8, c, acc[q][2] * (1.f - v.x * v.x), acc[q][3] * (1.f - v.y * v.y));
+    }
+}
+// Bias gradient: column sums of a hidden layer's delta.
+__device__ __forceinline__ void bias_grad(const __nv_bfloat16 *d, float *grad)
+{
+    if (threadIdx.x >= H) return;
+    float sum = 0.f;
+#pragma unroll
+    for (int s = 0; s < SAMPLES; ++s) sum += __bfloat162float(d[s * LD128 + threadIdx.x]);
+    atomicAdd(&grad[threadIdx.x], sum);
 }
 
 // Forward, mean-squared-error gradient, back-propagation and weight
 // gradients of the CTA's samples; gradients are added into grad (FP32, the
-// parameter layout) and the squared error into *loss.
-__global__ void __launch_bounds__(THREADS)
+// parameter layout) and, where it is wanted, the squared error into *loss.
+__global__ void __launch_bounds__(THREADS, 1)
     mlp_train_kernel(Params P, const float *X, int nin, const float *T, int nout,
                      int B, float *grad, float *loss)
 {
-    extern __shared__ __align__(16) unsigned char raw[];
-    Smem &S = *reinterpret_cast<Smem *>(raw);
-    const int s0 = blockIdx.x * SAMPLES, warp = threadIdx.x >> 5;
-    load_inputs(S, X, nin, B, s0);
-    forward(P, S);
-    // output delta: d(mean sq error)/dy = 2 (y - t) / (B nout)
-    float se = 0.f;
-    for (int q = threadIdx.x; q < SAMPLES * DOUT; q += THREADS) {
-        const int s = q / DOUT, c = q % DOUT, gs = s0 + s;
-        float d = 0.f;
-        if (gs < B && c < nout) {
-            const float e = S.out[q] - T[(long long)gs * nout + c];
-            se += e * e;
-            d = 2.f * e / (float)(B * nout);
-        }
-        const __nv_bfloat16 bd = __float2bfloat16(d);
-        S.dlt[s * DOUT + c] = bd;
-        S.dltT[c * SAMPLES + s] = bd;
-        if (c < DOUT) atomicAdd(&grad[b_off(NL - 1) + c], d);
-    }
-    for (int o = 16; o > 0; o >>= 1) se += __shfl_down_sync(0xffffffffu, se, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, se);
-    __syncthreads();
-    for (int l = NL - 1; l >= 0; --l) {
-        const int K = layer_k(l), N = layer_n(l);
-        // weight gradient dW[k][n] = sum_s act_l[s][k] dlt[s][n]:
-        // rows k (16 per warp-pass), contraction over the 64 samples
-        for (int kb = warp * 16; kb < K; kb += WARPS * 16) {
-            const __nv_bfloat16 *A = S.actT[l] + kb * SAMPLES;
-            if (N == H) {
-                float acc[H / 8][4] = {};
-                warp_gemm<SAMPLES, H>(A, SAMPLES, S.dltT, SAMPLES, acc);
-#pragma unroll
-                for (int j = 0; j < H / 8; ++j)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        int r, c;
-                        acc_pos(j, q, r, c);
-                        atomicAdd(&grad[w_off(l) + (kb + r) * N + c], acc[j][q]);
-                    }
-            } else {
-                float acc[DOUT / 8][4] = {};
-                warp_gemm<SAMPLES, DOUT>(A, SAMPLES, S.dltT, SAMPLES, acc);
-#pragma unroll
-                for (int j = 0; j < DOUT / 8; ++j)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        int r, c;
-                        acc_pos(j, q, r, c);
-                        atomicAdd(&grad[w_off(l) + (kb + r) * N + c], acc[j][q]);
-                    }
+    __shared__ __align__(16) Smem S;
+    Weights W;
+    Biases Bs;
+    const int warp = threadIdx.x >> 5;
+    after_predecessor();
+    load_weights<true>(P, W);
+    load_biases(P, Bs);
+    for (int s0 = blockIdx.x * SAMPLES; s0 < B; s0 += gridDim.x * SAMPLES) {
+        forward(W, Bs, S, X, nin, B, s0);
+        {   // output delta: d(mean sq error)/dy = 2 (y - t) / (B nout)
+            const int s = threadIdx.x / DOUT, c = threadIdx.x % DOUT, gs = s0 + s;
+            float d = 0.f, se = 0.f;
+            if (gs < B && c < nout) {
+                const float e = S.out[threadIdx.x] - T[(long long)gs * nout + c];
+                se = e * e;
+                d = 2.f * e / (float)(B * nout);
+            }
+            S.dout[s * LD16 + c] = __float2bfloat16(d);
+            d += __shfl_xor_sync(0xffffffffu, d, 16);  // the warp's two samples
+            if ((threadIdx.x & 16) == 0) atomicAdd(&grad[b_off(NL - 1) + c], d);
+            if (loss) {
+                for (int o = 16; o > 0; o >>= 1) se += __shfl_down_sync(0xffffffffu, se, o);
+                if ((threadIdx.x & 31) == 0) atomicAdd(loss, se);
             }
         }
-        if (l == 0) break;
-        // delta of the layer below: (dlt W^T) * (1 - a^2), a = act[l]
-        load_bt(S.wt, P.w + w_off(l), K * N);  // W [k][n]: Bt for this product
         __syncthreads();
-        float acc[H / 8][4] = {};
-        const __nv_bfloat16 *A = S.dlt + warp * 16 * N;
-        if (N == H) warp_gemm<H, H>(A, N, S.wt, N, acc);
-        else warp_gemm<DOUT, H>(A, N, S.wt, N, acc);
-        __syncthreads();  // every warp has read dlt and wt
-#pragma unroll
-        for (int j = 0; j < H / 8; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                int r, c;
-                acc_pos(j, q, r, c);
-                const int s = warp * 16 + r;
-                const float a = __bfloat162float(S.act[l][s * H + c]);
-                const float d = (s0 + s < B) ? acc[j][q] * (1.f - a * a) : 0.f;
-                const __nv_bfloat16 bd = __float2bfloat16(d);
-                S.dlt[s * H + c] = bd;
-                S.dltT[c * SAMPLES + s] = bd;
-            }
-        __syncthreads();
-        // bias gradient of layer l - 1: column sums of the new delta
-        for (int c = threadIdx.x; c < H; c += THREADS) {
-            float sum = 0.f;
-            for (int s = 0; s < SAMPLES; ++s) sum += __bfloat162float(S.dlt[s * H + c]);
-            atomicAdd(&grad[b_off(l - 1) + c], sum);
+        {
+            float acc[2][4] = {};
+            const FragA a = frag_a<LD16>(S.dout, 0);
+            mma(acc[0], a, W.b3[0].x, W.b3[0].y);
+            mma(acc[1], a, W.b3[1].x, W.b3[1].y);
+            hidden_delta(acc, S.act[2], S.dlt[0]);
         }
+        weight_grad<LD128, LD16, DOUT, 2>(S.act[2], S.dout, warp * 16, 0, grad + w_off(3));
         __syncthreads();
+        {
+            float acc[2][4] = {};
+            product<2>(S.dlt[0], W.b2, acc);
+            hidden_delta(acc, S.act[1], S.dlt[1]);
+        }
+        weight_grad<LD128, LD128, H, 16>(S.act[1], S.dlt[0], warp * 16, 0, grad + w_off(2));
+        bias_grad(S.dlt[0], grad + b_off(2));
+        __syncthreads();
+        {
+            float acc[2][4] = {};
+            product<2>(S.dlt[1], W.b1, acc);
+            // every warp has finished with the first delta (barrier above)
+            hidden_delta(acc, S.act[0], S.dlt[0]);
+        }
+        weight_grad<LD128, LD128, H, 16>(S.act[0], S.dlt[1], warp * 16, 0, grad + w_off(1));
+        bias_grad(S.dlt[1], grad + b_off(1));
+        __syncthreads();
+        weight_grad<LD16, LD128, H, 2>(S.in, S.dlt[0], 0, warp * 16, grad + w_off(0));
+        bias_grad(S.dlt[0], grad + b_off(0));
+        __syncthreads();  // the next samples reuse S
     }
 }
 
@@ -278,6 +418,7 @@ __global__ void mlp_adam_kernel(float *p, float *grad, float *m, float *v,
                                 float b1, float b2, float eps, float c1, float c2)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    after_predecessor();
     if (i >= NPARAM) return;
     const float g = grad[i];
     m[i] = b1 * m[i] + (1.f - b1) * g;
@@ -289,8 +430,9 @@ __global__ void mlp_adam_kernel(float *p, float *grad, float *m, float *v,
         while (l + 1 < NL && i >= w_off(l + 1)) ++l;
         const int K = layer_k(l), N = layer_n(l), local = i - w_off(l);
         const int k = local / N, n = local % N;
-        w[i] = __float2bfloat16(p[i]);
-        wt[w_off(l) + n * K + k] = __float2bfloat16(p[i]);
+        const __nv_bfloat16 b = __float2bfloat16(p[i]);
+        w[w_off(l) + frag_pos(k, n, N)] = b;
+        wt[w_off(l) + frag_pos(n, k, K)] = b;
     }
 }
 
@@ -328,20 +470,22 @@ lbm_status mfail(lbm_mlp *m, lbm_status s, const char *msg, cudaError_t e)
 
 Params params_of(const lbm_mlp *m) { return Params{m->wt, m->w, m->p}; }
 
-lbm_status smem_attr(lbm_mlp *m)
+int ctas(int B) { return std::min((B + SAMPLES - 1) / SAMPLES, MAX_CTAS); }
+
+// A launch that may start while its predecessor on the stream still runs
+// (the kernel waits for it, after_predecessor).
+template <class... K, class... A>
+cudaError_t launch_after(void (*kern)(K...), int grid, int block, A... args)
 {
-    static int configured = -1;
-    int dev = 0;
-    MCUDA(m, cudaGetDevice(&dev), "cudaGetDevice");
-    if (configured == dev) return LBM_OK;
-    MCUDA(m, cudaFuncSetAttribute(mlp_infer_kernel,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(Smem)), "mlp smem");
-    MCUDA(m, cudaFuncSetAttribute(mlp_train_kernel,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(Smem)), "mlp smem");
-    configured = dev;
-    return LBM_OK;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, K(args)...);
 }
 }  // namespace
 
@@ -398,23 +542,19 @@ lbm_status lbm_mlp_train(lbm_mlp *m, const float *X, int nin, const float *T,
         iters < 0 || !(lr >= 0))
         return mfail(m, LBM_ERR_ARG, "bad training arguments", cudaSuccess);
     MCUDA(m, cudaSetDevice(m->device), "cudaSetDevice");
-    lbm_status st = smem_attr(m);
-    if (st != LBM_OK) return st;
-    const int blocks = (B + SAMPLES - 1) / SAMPLES;
     float loss = 0.f;
+    MCUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float)), "memset");
     for (int it = 0; it < iters; ++it) {
-        MCUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float)), "memset");
-        mlp_train_kernel<<<blocks, THREADS, sizeof(Smem)>>>(params_of(m), X, nin,
-                                                           T, nout, B, m->grad,
-                                                           m->loss);
-        MCUDA(m, cudaGetLastError(), "mlp train launch");
+        // the error of the last forward pass is the one reported
+        MCUDA(m, launch_after(mlp_train_kernel, ctas(B), THREADS, params_of(m), X, nin, T, nout,
+                              B, m->grad, it + 1 == iters ? m->loss : nullptr),
+              "mlp train launch");
         ++m->steps;
         const float c1 = 1.f - std::pow(0.9f, (float)m->steps);
         const float c2 = 1.f - std::pow(0.999f, (float)m->steps);
-        mlp_adam_kernel<<<(NPARAM + 255) / 256, 256>>>(m->p, m->grad, m->m, m->v,
-                                                       m->wt, m->w, lr, 0.9f,
-                                                       0.999f, 1e-8f, c1, c2);
-        MCUDA(m, cudaGetLastError(), "mlp adam launch");
+        MCUDA(m, launch_after(mlp_adam_kernel, (NPARAM + 255) / 256, 256, m->p, m->grad, m->m,
+                              m->v, m->wt, m->w, lr, 0.9f, 0.999f, 1e-8f, c1, c2),
+              "mlp adam launch");
     }
     MCUDA(m, cudaMemcpy(&loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost),
           "loss copy");
@@ -430,14 +570,11 @@ lbm_status lbm_mlp_gradient(lbm_mlp *m, const float *X, int nin, const float *T,
     if (!X || !T || !grad || B <= 0 || nin < 1 || nin > DIN || nout < 1 || nout > DOUT)
         return mfail(m, LBM_ERR_ARG, "bad gradient arguments", cudaSuccess);
     MCUDA(m, cudaSetDevice(m->device), "cudaSetDevice");
-    lbm_status st = smem_attr(m);
-    if (st != LBM_OK) return st;
     // the training pass without the optimiser step: the accumulated full-batch
     // gradient is copied out and the accumulator cleared again
     MCUDA(m, cudaMemsetAsync(m->grad, 0, NPARAM * sizeof(float)), "memset");
     MCUDA(m, cudaMemsetAsync(m->loss, 0, sizeof(float)), "memset");
-    mlp_train_kernel<<<(B + SAMPLES - 1) / SAMPLES, THREADS, sizeof(Smem)>>>(
-        params_of(m), X, nin, T, nout, B, m->grad, m->loss);
+    mlp_train_kernel<<<ctas(B), THREADS>>>(params_of(m), X, nin, T, nout, B, m->grad, m->loss);
     MCUDA(m, cudaGetLastError(), "mlp gradient launch");
     float loss = 0.f;
     MCUDA(m, cudaMemcpy(grad, m->grad, NPARAM * sizeof(float), cudaMemcpyDeviceToHost),
@@ -457,10 +594,7 @@ lbm_status lbm_mlp_predict(lbm_mlp *m, const float *X, int nin, float *Y,
     if (!X || !Y || B <= 0 || nin < 1 || nin > DIN || nout < 1 || nout > DOUT)
         return mfail(m, LBM_ERR_ARG, "bad prediction arguments", cudaSuccess);
     MCUDA(m, cudaSetDevice(m->device), "cudaSetDevice");
-    lbm_status st = smem_attr(m);
-    if (st != LBM_OK) return st;
-    mlp_infer_kernel<<<(B + SAMPLES - 1) / SAMPLES, THREADS, sizeof(Smem)>>>(
-        params_of(m), X, nin, Y, nout, B);
+    mlp_infer_kernel<<<ctas(B), THREADS>>>(params_of(m), X, nin, Y, nout, B);
     MCUDA(m, cudaGetLastError(), "mlp infer launch");
     MCUDA(m, cudaDeviceSynchronize(), "mlp infer");
     return LBM_OK;
