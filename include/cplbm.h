@@ -88,9 +88,9 @@ typedef struct {
 
 /* Allocate a context and its device state for cfg.  *out receives the
  * context (NULL on error).  Device memory per lattice node: 8 distributions
- * in the storage type plus three densities; lattices that lbm_step can keep
- * on the chip (below) take 36 more values per node for the words their
- * tiles exchange. */
+ * in the storage type plus three densities; a lattice that lbm_step keeps
+ * on the chip (below) takes 36 more values per node, at its first such step,
+ * for the words its tiles exchange. */
 lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out);
 
 /* Select the equation of state (Sec. III): a, b, R as in Eqs. 16, 19, 22,

@@ -301,6 +301,28 @@ cudaError_t launch_one_step(lbm_ctx *c, cudaStream_t s)
                                : launch_step(c->L, p, p, s, &c->maps);
 }
 
+// The exchange words, at the first resident launch: contexts that never make
+// one do not hold them.  (Another stream of this thread may be capturing.)
+bool alloc_xchg(lbm_ctx *c)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+    const size_t bytes = xchg_bytes(c->L);
+    cudaError_t e = dev_alloc(&c->L.xchg, bytes);
+    // zero is no step's tag
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->L.xchg, 0, bytes, c->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        dev_free(c->L.xchg);
+        c->L.xchg = nullptr;
+    }
+#ifdef CPLBM_CHECK_BOUNDS
+    c->L.b_xchg = (long long)bytes;
+#endif
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return c->L.xchg != nullptr;
+}
+
 // Steps queued as resident launches (0 when they do not apply).
 int resident_steps(lbm_ctx *c, int left)
 {
@@ -311,6 +333,10 @@ int resident_steps(lbm_ctx *c, int left)
     if (c->stream && (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess ||
                       cs != cudaStreamCaptureStatusNone))
         return 0;
+    if (!c->L.xchg && !alloc_xchg(c)) {
+        c->resident = false;
+        return 0;
+    }
     int done = 0;
     while (left - done >= RESIDENT_MIN) {
         const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
@@ -466,16 +492,8 @@ lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
     alloc((void **)&c->d_prev, (size_t)L.nx * L.ny * sizeof(double));
     const char *no_tma = getenv("CPLBM_NO_TMA");
     c->use_tma = !(no_tma && no_tma[0] == '1');
-    if (alone && c->use_tma && st == LBM_OK && resident_plan(&L, 1, c->device, &c->plan)) {
-        alloc(&L.xchg, xchg_bytes(L));
-        c->resident = st == LBM_OK;
-#ifdef CPLBM_CHECK_BOUNDS
-        L.b_xchg = (long long)xchg_bytes(L);
-#endif
-        // zero is no step's tag
-        if (c->resident && cudaMemsetAsync(L.xchg, 0, xchg_bytes(L), c->stream) != cudaSuccess)
-            st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
-    }
+    c->resident = alone && c->use_tma && st == LBM_OK &&
+                  resident_plan(&L, 1, c->device, &c->plan);
     // the densities' row padding is loaded with the tiles and never written:
     // zero, once
     for (int k = 0; k < 2 && st == LBM_OK; ++k)
