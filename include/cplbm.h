@@ -114,7 +114,8 @@ lbm_status lbm_set_wall_mu(lbm_ctx *ctx, double mu_bottom, int top_mode,
  * (lbm_autotune chooses between the two).  The shape
  * changes speed, and in FP32 arithmetic the rounding order of some sums,
  * not the method.  May be called at any time.  Default: 64x16 (two nodes
- * per lane) for FP32 arithmetic, 32x32 for FP64. */
+ * per lane) for FP32 arithmetic (64x32 in FP32 storage where that leaves the
+ * last tile row higher than three rows and 64x16 does not), 32x32 for FP64. */
 lbm_status lbm_set_tile(lbm_ctx *ctx, int tx, int ty);
 lbm_status lbm_get_tile(const lbm_ctx *ctx, int *tx, int *ty);
 
@@ -365,7 +366,8 @@ lbm_status lbm_eos_pressure(int eos, double a, double b, double R,
  * TMA or cp.async interior path), 1 for an edge tile (the TMA paths only:
  * its halo wraps around a periodic edge or meets a wall, or, on 32-wide
  * shapes, it is the ragged last tile, at least 4 nodes wide, of a periodic
- * direction), 0 for a general tile, with ntx = ceil(nx / tx), nty =
+ * direction), 0 for a general tile (64-wide: also that ragged last tile,
+ * which a lattice by itself steps on the TMA path too), with ntx = ceil(nx / tx), nty =
  * ceil(fluid rows / ty) and max >= ntx * nty entries in kinds (a host
  * array).  seams != 0 gives the classes of a lattice (single or in a
  * batch) whose shape has a TMA path; seams == 0 those of a shape without

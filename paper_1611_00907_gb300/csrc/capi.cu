@@ -467,7 +467,7 @@ lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
     L.precision = cfg->precision;
     L.top_mode = 0;
     set_consts(L);
-    step_default_shape(L.precision, &L.tx, &L.ty);
+    step_default_shape(L, &L.tx, &L.ty);
 
     const size_t pb = pop_bytes(L.precision), rb = rho_bytes(L.precision);
     lbm_status st = LBM_OK;
@@ -723,7 +723,7 @@ lbm_status lbm_autotune(lbm_ctx *c, int nsteps, int *best_tx, int *best_ty)
     // where the lattice has a plan for the resident steps they are timed
     // beside the shapes (as shape index n, on the default shape)
     const bool can_stay = !c->plan.tiles.empty() && c->force_model == 0;
-    if (can_stay && n < 16) step_default_shape(L.precision, &tx[n], &ty[n]);
+    if (can_stay && n < 16) step_default_shape(L, &tx[n], &ty[n]);
     lbm_status st = snapshot(c, snap, true);
     cudaError_t e = cudaSuccess;
     if (st == LBM_OK) e = cudaEventCreate(&e0);

@@ -193,7 +193,7 @@ cudaError_t launch_step(const Lattice &L, int parity, int cur,
 // Whether the step has a kernel for tile shape tx x ty in precision prec,
 // and the default shape of a precision.
 bool step_shape_supported(int prec, int tx, int ty);
-void step_default_shape(int prec, int *tx, int *ty);
+void step_default_shape(const Lattice &L, int *tx, int *ty);
 // The compiled tile shapes, in a fixed order: returns how many, fills up to
 // `max` pairs.
 int step_shapes(int *tx, int *ty, int max);
@@ -214,9 +214,12 @@ bool pt_shape_supported(int prec, int tx, int ty);
 // least three full tiles span the lattice, and the last tile across the
 // edge is full or at least 4 nodes wide, so the halo that wraps around the
 // edge has the layout of an interior halo.  That ragged last tile takes the
-// TMA path too on 32-wide tiles (bit 3), whose tile function places the
-// right and top tile edges at the tile's own width and height; the
-// two-nodes-per-lane path leaves it to the general path.  Walls: at least
+// TMA path too with bit 3, its right and top edges at the tile's own width
+// and height: on 32-wide tiles always, on 64-wide ones in the single-lattice
+// kernels with the ragged variant (ragged_seam; batches keep such tiles on the
+// general path or, by default, take 32-wide tiles: an uneven batch of 32
+// lattices, sides 64 to 1024, ran at 108 us a step on 32 x 32, 122 on 64 x 16
+// with ragged tiles on the TMA path).  Walls: at least
 // two tile rows, the bottom one full and the one above it full or at least
 // 4 rows high, so the bottom wall tile's halo above sees interior tile
 // edges; the top wall tile may be ragged down to two rows (tile_kind).
@@ -229,6 +232,14 @@ __host__ __device__ inline int seam_bits(const Lattice &L, int tx, int ty)
     if (L.walls && (nfy >= 2 || (nfy == 1 && ry >= 4))) s |= 4;
     if (tx == 32) s |= 8;
     return s;
+}
+
+// Whether the last tile of a periodic direction that `seams` (seam_bits)
+// allows on a TMA path is ragged: on 64-wide shapes that takes the kernels
+// with the ragged variant of the two-nodes-per-lane path, and seam bit 3.
+inline bool ragged_seam(const Lattice &L, int tx, int ty, int seams)
+{
+    return (L.nx % tx != 0 && (seams & 1)) || (!L.walls && L.nyf % ty != 0 && (seams & 2));
 }
 
 // Path class of tile (bx, by): TILE_INTERIOR when the tile is full, its

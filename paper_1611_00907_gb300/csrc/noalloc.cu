@@ -216,7 +216,7 @@ extern "C" lbm_status lbm_step_noalloc(
     L.precision = P_F64;
     L.wait_cycles = WAIT_CYCLES_DEFAULT;  // no TMA path here; set for completeness
     set_consts(L);
-    step_default_shape(P_F64, &L.tx, &L.ty);
+    step_default_shape(L, &L.tx, &L.ty);
 
     if (cfg->device < 0 || cfg->device >= kMaxDevices)
         return fail_msg(LBM_ERR_ARG, "device ordinal %d out of range",

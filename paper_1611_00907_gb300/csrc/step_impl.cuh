@@ -1467,8 +1467,13 @@ struct TmaPairSmem {
                   "pair-aligned sub-arrays");
 };
 
-// PT: the baseline force of Eq. 5, as for step_tile_tma.
-template <class S, int TX, int TY, int NT, int PARITY, int EDGE, bool PT = false>
+// PT: the baseline force of Eq. 5, as for step_tile_tma.  RAG: the variant of
+// edge tiles that may be the ragged last tile of a periodic direction, hx
+// columns and hy rows of it in use (as step_tile_tma); a pair may then have
+// its second node beyond the lattice.  Only kernels of lattices with such
+// tiles hold it.
+template <class S, int TX, int TY, int NT, int PARITY, int EDGE, bool PT = false,
+          bool RAG = false>
 __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, int X0,
                                                    int Y0, unsigned char *smem_raw,
                                                    TileMaps maps,
@@ -1497,6 +1502,7 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
     // wraps around a periodic edge, of a periodic lattice (1) or of any
     // lattice, walls included (2)
     constexpr bool seam = EDGE != 0, walls_ok = EDGE == 2;
+    static_assert(!RAG || seam, "ragged tiles are edge tiles");
 
     // 1. Loads (bar, phase, seam tiles: as step_tile_tma).
     if (threadIdx.x == 0) {
@@ -1528,10 +1534,11 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
 
     // 2. Partial sums into the halo's tile-edge nodes (order of
     //    load_rho_stored); halo (lx, ly) is staged at row ly, column lx + 2.
-    combine_ring<float, TX, TY, NT, RP>(s_rho, s_ring, TX, TY);
+    const SeamEdges edge = seam_edges<walls_ok>(L, X0, Y0, TX, TY);
+    const int hx = RAG ? edge.hx : TX;
+    combine_ring<float, TX, TY, NT, RP>(s_rho, s_ring, hx, RAG ? edge.hy : TY);
     __syncthreads();
     // edge tiles at a wall: the solid row's density (Eq. 28)
-    const SeamEdges edge = seam_edges<walls_ok>(L, X0, Y0, TX, TY);
     if (walls_ok) wall_rho_rows<float, TX, NT, RP>(edge, s_rho);
 
     // 3. mu at halo column a (x = X0 - 1 + a) and row b (r = Y0 - 1 + b),
@@ -1630,9 +1637,15 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
     for (int i = 1; i < 9; ++i)
         woff[i] = PARITY == 0 ? (opp(i) - 1) * (int)L.plane
                               : (i - 1) * (int)L.plane + ey(i) * L.pitch + ex(i);
-    // wall tiles: rows 0 .. hy - 1 hold fluid (as step_tile_tma)
-    const int hy = walls_ok ? edge.hy : TY;
-    const bool has_l = lane > 0, has_r = lane < 31;
+    // wall and ragged tiles: rows 0 .. hy - 1 hold fluid (as step_tile_tma),
+    // columns 0 .. hx - 1 belong to the tile; lane lr holds the last one, in
+    // its second node when lr_y
+    constexpr bool part_y = walls_ok || RAG;
+    const int hy = part_y ? edge.hy : TY;
+    const int lr = RAG ? (hx - 1) >> 1 : 31;
+    const bool lr_y = !RAG || (hx & 1) == 0;
+    const bool ok0 = !RAG || x0 < hx, ok1 = !RAG || x0 + 1 < hx;  // nodes of the tile
+    const bool has_l = lane > 0, has_r = RAG ? x0 + 2 < hx : lane < 31;
     // windows: density of tile row ly at staged row ly + 2, column x0 + 4;
     // mu of tile row ly at s_mu row ly + 1, column x0 + 2
     Row2 rd = row2(s_rho, (ly0 + 1) * RP + x0 + 4), rm = row2(s_rho, (ly0 + 2) * RP + x0 + 4);
@@ -1647,8 +1660,10 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
     }
     float2 pend = p2(0.0f), up_prev = p2(0.0f), first = p2(0.0f);
     float pend_c = 0.0f, up_prev_c = 0.0f, first_c = 0.0f;
-    const int slot_c = TX + (lane == 31);        // exchange slot of a column
-    const int xc = lane == 0 ? X0 - 1 : X0 + TX;  // ring column of the lane
+    float2 up_top = p2(0.0f);  // RAG: "up" of the tile's last row hy - 1
+    float up_top_c = 0.0f;
+    const int slot_c = TX + (lane == lr);        // exchange slot of a column
+    const int xc = lane == 0 ? X0 - 1 : X0 + hx;  // ring column of the lane
     const int cls_c = lane == 0 ? R_R : R_L;
     // this tile, and the tile of the ring column a lane feeds (classes L and
     // R share one index layout)
@@ -1656,12 +1671,28 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
     const int bxl = neighbour_tile(X0, -1, TX, L.nx, seam), bxr = neighbour_tile(X0, 1, TX, L.nx, seam);
     const int byb = neighbour_tile(Y0, -1, TY, L.nyf, seam), byt = neighbour_tile(Y0, 1, TY, L.nyf, seam);
     const int bxc = lane == 0 ? bxl : bxr;
-    const bool col_lane = lane == 0 || lane == 31;
+    const bool col_lane = lane == 0 || lane == lr;
+    // a pair of values, or its first where the second node is not the tile's
+    auto put_pair = [&](float *q, float2 v, bool in) {
+        if (!in) return;
+        if (ok1) *reinterpret_cast<float2 *>(q) = v;
+        else if (ok0) *q = v.x;
+    };
+    auto put_rho2 = [&](long long row, float2 v) {
+        float *q = (float *)Rn + row * L.pitch + X0 + x0;
+        put_pair(q, v, ok0 && CPLBM_IN_RHO(L, nxt, q, ok1 ? 2 : 1));
+    };
+    auto put_ring2 = [&](int c, long long idx, float2 v) {
+        float *q = (float *)ring[c] + idx;
+        put_pair(q, v, ok0 && CPLBM_IN_RING(L, nxt, c, q, ok1 ? 2 : 1));
+    };
     pop_t *Arow = A + (long long)(Y0 + ly0) * L.pitch + X0 + x0;
     // corrections of odd-step write offsets across the periodic edges
     const int wrap_y = L.nyf * L.pitch;
     const int cxl = (PARITY == 1 && seam && X0 == 0 && lane == 0) ? L.nx : 0;
-    const int cxr = (PARITY == 1 && seam && X0 + TX >= L.nx && lane == 31) ? -L.nx : 0;
+    const bool last_x = PARITY == 1 && seam && X0 + TX >= L.nx;
+    const int cxr = last_x && lane == lr && lr_y ? -L.nx : 0;
+    const int cxr0 = RAG && last_x && lane == lr && !lr_y ? -L.nx : 0;  // first node
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int ly = ly0 + k;
@@ -1674,7 +1705,7 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
         }
         float2 same = p2(0.0f), up = p2(0.0f), down = p2(0.0f);
         float same_c = 0.0f, up_c = 0.0f, down_c = 0.0f;
-        if (!walls_ok || ly < hy) {  // warp-uniform
+        if (!part_y || ly < hy) {  // warp-uniform
             float2 f[9];
 #pragma unroll
             for (int i = 1; i < 9; ++i) {
@@ -1712,7 +1743,7 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
                 // are stored one node at a time); a population heading into a
                 // solid row goes to the node's own slot opp(i)
                 const int cyb = (PARITY == 1 && seam && edge.yb && ly == 0) ? wrap_y : 0;
-                const int cyt = (PARITY == 1 && seam && edge.yt && ly == TY - 1) ? -wrap_y : 0;
+                const int cyt = (PARITY == 1 && seam && edge.yt && ly == hy - 1) ? -wrap_y : 0;
 #pragma unroll
                 for (int i = 1; i < 9; ++i) {
                     const bool into_wall = PARITY == 1 && ((ey(i) < 0 && wall_b) ||
@@ -1720,11 +1751,15 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
                     pop_t *dst = into_wall ? Arow + (opp(i) - 1) * (int)L.plane
                                            : Arow + woff[i] + (ey(i) < 0 ? cyb : ey(i) > 0 ? cyt : 0);
                     if (PARITY == 0 || ex(i) == 0 || into_wall) {
-                        if (CPLBM_IN_POPS(L, dst, 2)) st_pair(dst, fp[i]);
+                        if (ok1) {
+                            if (CPLBM_IN_POPS(L, dst, 2)) st_pair(dst, fp[i]);
+                        } else if (ok0) {
+                            if (CPLBM_IN_POPS(L, dst, 1)) st_real(dst, fp[i].x);
+                        }
                     } else {
-                        pop_t *d0 = dst + (ex(i) < 0 ? cxl : 0), *d1 = dst + 1 + (ex(i) > 0 ? cxr : 0);
-                        if (CPLBM_IN_POPS(L, d0, 1)) st_real(d0, fp[i].x);
-                        if (CPLBM_IN_POPS(L, d1, 1)) st_real(d1, fp[i].y);
+                        pop_t *d0 = dst + (ex(i) < 0 ? cxl : cxr0), *d1 = dst + 1 + (ex(i) > 0 ? cxr : 0);
+                        if (ok0 && CPLBM_IN_POPS(L, d0, 1)) st_real(d0, fp[i].x);
+                        if (ok1 && CPLBM_IN_POPS(L, d1, 1)) st_real(d1, fp[i].y);
                     }
                 }
             }
@@ -1736,24 +1771,28 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
             const float f3r = __shfl_down_sync(0xffffffffu, fp[3].x, 1);
             const float f6r = __shfl_down_sync(0xffffffffu, fp[6].x, 1);
             const float f7r = __shfl_down_sync(0xffffffffu, fp[7].x, 1);
-            same = make_float2((fp[0].x + (has_l ? f1l : 0.0f)) + fp[3].y,
+            same = make_float2((fp[0].x + (has_l ? f1l : 0.0f)) + (ok1 ? fp[3].y : 0.0f),
                                (fp[0].y + fp[1].x) + (has_r ? f3r : 0.0f));
-            up = make_float2((fp[2].x + (has_l ? f5l : 0.0f)) + fp[6].y,
+            up = make_float2((fp[2].x + (has_l ? f5l : 0.0f)) + (ok1 ? fp[6].y : 0.0f),
                              (fp[2].y + fp[5].x) + (has_r ? f6r : 0.0f));
-            down = make_float2((fp[4].x + (has_l ? f8l : 0.0f)) + fp[7].y,
+            down = make_float2((fp[4].x + (has_l ? f8l : 0.0f)) + (ok1 ? fp[7].y : 0.0f),
                                (fp[4].y + fp[8].x) + (has_r ? f7r : 0.0f));
             // what leaves into a solid row comes back to the node
             if (wall_b) same = padd(same, padd(padd(fp[4], fp[7]), fp[8]));
             if (wall_t) same = padd(same, padd(padd(fp[2], fp[5]), fp[6]));
             // ring columns: lane 0 feeds x = X0 - 1 (f*_3; f*_6 up; f*_7 down)
-            // from its first node, lane 31 feeds x = X0 + TX (f*_1; f*_5 up;
-            // f*_8 down) from its second
-            same_c = lane == 0 ? fp[3].x : fp[1].y;
-            up_c = lane == 0 ? fp[6].x : fp[5].y;
-            down_c = lane == 0 ? fp[7].x : fp[8].y;
+            // from its first node, lane lr feeds x = X0 + hx (f*_1; f*_5 up;
+            // f*_8 down) from the tile's last column
+            same_c = lane == 0 ? fp[3].x : lr_y ? fp[1].y : fp[1].x;
+            up_c = lane == 0 ? fp[6].x : lr_y ? fp[5].y : fp[5].x;
+            down_c = lane == 0 ? fp[7].x : lr_y ? fp[8].y : fp[8].x;
+        }
+        if (RAG && ly == hy - 1) {
+            up_top = up;
+            up_top_c = up_c;
         }
         Arow += L.pitch;
-        const bool row_ok = !walls_ok || ly - 1 < hy;
+        const bool row_ok = !part_y || ly - 1 < hy;
         if (k == 0) {
             *reinterpret_cast<float2 *>(s_down + warp * XW + x0) = down;
             if (col_lane) s_down[warp * XW + slot_c] = down_c;
@@ -1766,7 +1805,7 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
                 first = done;
                 first_c = done_c;
             } else if (row_ok) {
-                put_rho(L, nxt, Rn, (long long)(Y0 + ly - 1) * L.pitch + X0 + x0, done);
+                put_rho2(Y0 + ly - 1, done);
                 if (col_lane) put_ring(L, nxt, ring, cls_c, ring_index(L, R_L, bxc, by, Y0 + ly - 1, xc), done_c);
             }
             pend = padd(same, up_prev);
@@ -1795,30 +1834,32 @@ __device__ __forceinline__ bool step_tile_tma_pair(const Lattice &L, int cur, in
             top = padd(top, *reinterpret_cast<const float2 *>(s_down + (warp + 1) * XW + x0));
             top_c += s_down[(warp + 1) * XW + slot_c];
         }
-        if (!walls_ok || ly0 + PER - 1 < hy) {
-            put_rho(L, nxt, Rn, (long long)(Y0 + ly0 + PER - 1) * L.pitch + X0 + x0, top);
+        if (!part_y || ly0 + PER - 1 < hy) {
+            put_rho2(Y0 + ly0 + PER - 1, top);
             if (col_lane) put_ring(L, nxt, ring, cls_c, ring_index(L, R_L, bxc, by, Y0 + ly0 + PER - 1, xc), top_c);
         }
         if (warp > 0) {
             first = padd(first, *reinterpret_cast<const float2 *>(s_up + (warp - 1) * XW + x0));
             first_c += s_up[(warp - 1) * XW + slot_c];
         }
-        if (!walls_ok || ly0 < hy) {
-            put_rho(L, nxt, Rn, (long long)(Y0 + ly0) * L.pitch + X0 + x0, first);
+        if (!part_y || ly0 < hy) {
+            put_rho2(Y0 + ly0, first);
             if (col_lane) put_ring(L, nxt, ring, cls_c, ring_index(L, R_L, bxc, by, Y0 + ly0, xc), first_c);
         }
     }
     // ring rows below and above the tile, with their corners (none across a
     // wall)
     if (warp == 0 && !(walls_ok && edge.wb)) {
-        put_ring(L, nxt, ring, R_T, ring_index(L, R_T, bx, byb, Y0 - 1, X0 + x0), *reinterpret_cast<const float2 *>(s_down + x0));
+        put_ring2(R_T, ring_index(L, R_T, bx, byb, Y0 - 1, X0 + x0), *reinterpret_cast<const float2 *>(s_down + x0));
         if (lane == 0) put_ring(L, nxt, ring, R_TR, ring_index(L, R_TR, bxl, byb, Y0 - 1, X0 - 1), s_down[TX]);
-        if (lane == 31) put_ring(L, nxt, ring, R_TL, ring_index(L, R_TL, bxr, byb, Y0 - 1, X0 + TX), s_down[TX + 1]);
+        if (lane == lr) put_ring(L, nxt, ring, R_TL, ring_index(L, R_TL, bxr, byb, Y0 - 1, X0 + hx), s_down[TX + 1]);
     }
-    if (warp == NW - 1 && !(walls_ok && edge.wt)) {
-        put_ring(L, nxt, ring, R_B, ring_index(L, R_B, bx, byt, Y0 + TY, X0 + x0), up_prev);
-        if (lane == 0) put_ring(L, nxt, ring, R_BR, ring_index(L, R_BR, bxl, byt, Y0 + TY, X0 - 1), up_prev_c);
-        if (lane == 31) put_ring(L, nxt, ring, R_BL, ring_index(L, R_BL, bxr, byt, Y0 + TY, X0 + TX), up_prev_c);
+    const float2 upt = RAG ? up_top : up_prev;
+    const float upt_c = RAG ? up_top_c : up_prev_c;
+    if (warp == (RAG ? (hy - 1) / PER : NW - 1) && !(walls_ok && edge.wt)) {
+        put_ring2(R_B, ring_index(L, R_B, bx, byt, Y0 + hy, X0 + x0), upt);
+        if (lane == 0) put_ring(L, nxt, ring, R_BR, ring_index(L, R_BR, bxl, byt, Y0 + hy, X0 - 1), upt_c);
+        if (lane == lr) put_ring(L, nxt, ring, R_BL, ring_index(L, R_BL, bxr, byt, Y0 + hy, X0 + hx), upt_c);
     }
     return true;
 }
@@ -1860,8 +1901,10 @@ constexpr int pair_min_ctas()
 
 // WALLS: the kernel of walled lattices, whose edge tiles include the wall
 // rows; periodic lattices take the variant without the wall code, so that it
-// does not weigh on the code the interior tiles run.
-template <class S, int TX, int TY, int NT, int PARITY, bool WALLS>
+// does not weigh on the code the interior tiles run.  RAG (two-nodes-per-lane
+// shapes): likewise the kernel of lattices whose last tile of a periodic
+// direction is ragged (launch_shape).
+template <class S, int TX, int TY, int NT, int PARITY, bool WALLS, bool RAG>
 __global__ void __launch_bounds__(NT, HasTmaPair<S, TX, TY, NT>::value
                                           ? pair_min_ctas<S, TX, TY, NT>() : 0)
     step_kernel(const Lattice L, int cur, int seams, const __grid_constant__ TmaMaps maps)
@@ -1897,7 +1940,7 @@ __global__ void __launch_bounds__(NT, HasTmaPair<S, TX, TY, NT>::value
                     step_tile_tma_pair<S, TX, TY, NT, PARITY, 0>(L, cur, X0, Y0,
                                                                  smem_raw, tm, bar, 0);
                 else
-                    step_tile_tma_pair<S, TX, TY, NT, PARITY, WALLS ? 2 : 1>(
+                    step_tile_tma_pair<S, TX, TY, NT, PARITY, WALLS ? 2 : 1, false, RAG>(
                         L, cur, X0, Y0, smem_raw, tm, bar, 0);
             }
             return;
@@ -1923,41 +1966,49 @@ static cudaError_t launch_shape(const Lattice &L, int parity, int cur,
     const size_t smem_max = smem_v4 > smem_tma ? smem_v4 : smem_tma;
     TmaMaps m{};
     if (maps && maps->valid && maps->tx == TX && maps->ty == TY) m = *maps;
-    // kernels of periodic (index 0) and walled (1) lattices, by parity
-    void (*const kern[2][2])(const Lattice, int, int, const TmaMaps) = {
-        {step_kernel<S, TX, TY, NT, 0, false>, step_kernel<S, TX, TY, NT, 1, false>},
-        {step_kernel<S, TX, TY, NT, 0, true>, step_kernel<S, TX, TY, NT, 1, true>}};
+    // Tile classes (tile_kind): the TMA paths also take the seam tiles of
+    // periodic edges.  A lattice whose sides are no multiples of a 64-wide
+    // tile takes the kernel whose edge tiles may be ragged, unless what is
+    // left over is too narrow for it (seam_bits); 1001 x 757 FP32 offset: 25.0
+    // -> 16.4 us a step against those tiles on the general path.
+    const int ntx = (L.nx + TX - 1) / TX, nty = (L.nyf + TY - 1) / TY;
+    const int rx = L.nx % TX, ry = L.nyf % TY;
+    int seams = HasTma<S, TX, TY, NT>::value || HasTmaPair<S, TX, TY, NT>::value
+                    ? seam_bits(L, TX, TY) : 0;
+    const bool rag = HasTmaPair<S, TX, TY, NT>::value && m.valid &&
+                     ragged_seam(L, TX, TY, seams);
+    if (rag) seams |= 8;
+    // kernels by ragged last tiles, walls and parity
+    constexpr bool R = HasTmaPair<S, TX, TY, NT>::value;  // others: one kernel for both
+    void (*const kern[2][2][2])(const Lattice, int, int, const TmaMaps) = {
+        {{step_kernel<S, TX, TY, NT, 0, false, false>, step_kernel<S, TX, TY, NT, 1, false, false>},
+         {step_kernel<S, TX, TY, NT, 0, true, false>, step_kernel<S, TX, TY, NT, 1, true, false>}},
+        {{step_kernel<S, TX, TY, NT, 0, false, R>, step_kernel<S, TX, TY, NT, 1, false, R>},
+         {step_kernel<S, TX, TY, NT, 0, true, R>, step_kernel<S, TX, TY, NT, 1, true, R>}}};
     static int configured = -1;  // device the attributes were set on
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (configured != dev) {
-        for (int w = 0; w < 2 && e == cudaSuccess; ++w)
-            for (int p = 0; p < 2 && e == cudaSuccess; ++p)
-                e = cudaFuncSetAttribute(kern[w][p],
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_max);
+        for (int q = 0; q < 8 && e == cudaSuccess; ++q)
+            e = cudaFuncSetAttribute(kern[q >> 2][q >> 1 & 1][q & 1],
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem_max);
         if (e != cudaSuccess) return e;
         configured = dev;
     }
-    // Tile classes (tile_kind): the TMA paths also take the seam tiles of
-    // periodic edges.
-    const int ntx = (L.nx + TX - 1) / TX, nty = (L.nyf + TY - 1) / TY;
-    const int seams = HasTma<S, TX, TY, NT>::value || HasTmaPair<S, TX, TY, NT>::value
-                          ? seam_bits(L, TX, TY) : 0;
     // When every tile is interior or an edge tile and the maps are valid,
     // every tile takes the TMA path (step_kernel has no general fallback on
     // it), so the launch needs only that path's shared memory, and more CTAs
-    // fit: x periodic seams over full tiles, and in y either periodic seams
-    // over full tiles or walls whose top tile is full or at least 4 rows
-    // high (otherwise the tile below it is general).
-    const int ry = L.nyf % TY;
-    const bool all_tma = m.valid && (seams & 1) && L.nx % TX == 0 &&
+    // fit: x periodic seams over full tiles (or ragged ones where the path
+    // takes them), and in y the same or walls whose top tile is full or at
+    // least 4 rows high (otherwise the tile below it is general).
+    const bool all_tma = m.valid && (seams & 1) && (rx == 0 || rag) &&
                          (L.walls ? ((seams & 4) && (ry == 0 || ry >= 4))
-                                  : ((seams & 2) && ry == 0));
+                                  : ((seams & 2) && (ry == 0 || rag)));
     const size_t smem = (all_tma && smem_tma > 0) ? smem_tma : smem_max;
     dim3 grid(ntx, nty);
-    kern[L.walls ? 1 : 0][parity & 1]<<<grid, NT, smem, s>>>(L, cur, seams, m);
+    kern[rag][L.walls ? 1 : 0][parity & 1]<<<grid, NT, smem, s>>>(L, cur, seams, m);
     return cudaGetLastError();
 }
 
