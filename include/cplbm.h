@@ -150,7 +150,7 @@ lbm_status lbm_init(lbm_ctx *ctx, const double *rho, const double *ux,
 /* Queue nsteps (>= 0) time steps (Sec. II: density, Eq. 8, Eq. 12, the
  * BGK collision of Eq. 13-14 and streaming, with the wall rule of Sec. IV)
  * on the context's stream.  Returns without waiting for the GPU.  Four steps
- * or more of a lattice whose state fits the shared memory of all SMs together
+ * or more (24 in FP32 storage above 100 000 nodes) of a lattice whose state fits the shared memory of all SMs together
  * (FP64 up to about 270 000 nodes, FP32 storage about 500 000; not FP16, the
  * pressure-tensor force or a chosen tile shape) run as one cooperative launch
  * that keeps the state there; such launches follow one another on a device.
@@ -227,7 +227,7 @@ lbm_status lbm_batch_create(const lbm_instance *inst, int count, int precision,
 lbm_status lbm_batch_init(lbm_batch *b, int index, const double *rho,
                           const double *ux, const double *uy, int on_device);
 /* Queue nsteps steps of every active lattice; all must be initialised.  Four
- * steps or more of lattices that together fit the shared memory of all SMs
+ * steps or more (24, as for lbm_step) of lattices that together fit the shared memory of all SMs
  * run on the chip, as lbm_step's (not after lbm_batch_set_tile or
  * lbm_batch_schedule with a schedule). */
 lbm_status lbm_batch_step(lbm_batch *b, int nsteps);

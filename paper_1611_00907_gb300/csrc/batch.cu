@@ -149,7 +149,7 @@ lbm_status plan_resident(lbm_batch *b, std::vector<Lattice> &lats)
 int resident_steps(lbm_batch *b, int left)
 {
     int done = 0;
-    while (!b->plan.tiles.empty() && left - done >= RESIDENT_MIN) {
+    while (!b->plan.tiles.empty() && left - done >= b->plan.min_steps) {
         const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
         if (launch_resident(b->plan, nullptr, b->d_lats, b->d_tiles, n, (int)(b->t & 1),
                             b->xchg_tag, b->stream) != cudaSuccess) {

@@ -326,7 +326,7 @@ bool alloc_xchg(lbm_ctx *c)
 // Steps queued as resident launches (0 when they do not apply).
 int resident_steps(lbm_ctx *c, int left)
 {
-    if (!c->resident || c->force_model != 0 || left < RESIDENT_MIN) return 0;
+    if (!c->resident || c->force_model != 0 || left < c->plan.min_steps) return 0;
     // a caller's capture takes plain launches: the words' tags are good for
     // one run only
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -338,7 +338,7 @@ int resident_steps(lbm_ctx *c, int left)
         return 0;
     }
     int done = 0;
-    while (left - done >= RESIDENT_MIN) {
+    while (left - done >= c->plan.min_steps) {
         const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
         if (launch_resident(c->plan, &c->L, nullptr, nullptr, n, (int)(c->t & 1), c->xchg_tag,
                             c->stream) != cudaSuccess) {

@@ -25,8 +25,7 @@ size_t tile_smem(int prec, int w, int h)
     return rho_bytes(prec) * (size_t)Geo(w, h).elems();
 }
 
-// Threads of a CTA: enough for the nodes (FP32: pairs) of a w x h tile and
-// its rim, at most 512.
+// Threads of a CTA: 256 while every node and every two rim nodes have one.
 int rim_nodes(bool walls, int w, int h)
 {
     const int side = walls ? HX : RIM;
@@ -34,8 +33,8 @@ int rim_nodes(bool walls, int w, int h)
 }
 int threads_for(const Lattice &L, int w, int h)
 {
-    const int items = L.precision == P_F64 ? w * h : (w + 2) * (h + 3) / 2;
-    return items > 288 || rim_nodes(L.walls != 0, w, h) > 256 * RIM_NODES ? 512 : 256;
+    return w * h > 256 || rim_nodes(L.walls != 0, w, h) > 256 * RIM_NODES
+               ? resident_threads(L.precision == P_F64) : 256;
 }
 
 // Cost of a step of a w x h tile on one SM.  FP64: instructions per node of
@@ -68,7 +67,7 @@ bool cut(const Lattice &L, int most, int *w, int *h)
         while (L.walls && ny % hh == 1) ++hh;
         const int tw = std::min(ww, nx);
         if (tile_smem(prec, tw, hh) > RESIDENT_SMEM ||
-            rim_nodes(L.walls != 0, tw, hh) > 512 * RIM_NODES)
+            rim_nodes(L.walls != 0, tw, hh) > resident_threads(prec == P_F64) * RIM_NODES)
             continue;
         const double c = tile_cost(prec, tw, hh);
         if (best < 0 || c < best) {
@@ -175,6 +174,7 @@ bool resident_plan(const Lattice *lats, int count, int device, ResidentPlan *p)
     p->w = w[0];
     p->h = h[0];
     p->gx = (lats[0].nx + w[0] - 1) / w[0];
+    p->min_steps = resident_min(prec, nodes);
     p->device = device;
     p->precision = prec;
     return (int)p->tiles.size() <= sms;

@@ -25,14 +25,24 @@ struct ResidentArgs {
     unsigned tag;         // tag of the first step's exchange words
 };
 
-// A call of at least RESIDENT_MIN steps takes resident launches where there
-// is a plan for them; a launch takes at most RESIDENT_MAX, so that no kernel
-// holds the GPU for long.
-constexpr int RESIDENT_MIN = 4, RESIDENT_MAX = 4096;
+// A call takes resident launches from this many steps on, where there is a
+// plan for them.  Loading and storing the state costs 13 us (64 x 64) to 40 us
+// (500 x 500) a call, the step saves 20 us (FP32 64 x 64), 5 us (FP32 256 x
+// 256) or 18 us (FP64 500 x 500), but only 2 us for FP32 512 x 512: calls of 4
+// steps are faster throughout in FP64 and up to 100 000 nodes in FP32 (20 us
+// against 98 for 64 x 64, 28 against 43 for 256 x 256), larger FP32 lattices
+// break even at about 20.
+inline int resident_min(int prec, long long nodes)
+{
+    return prec == P_F64 || nodes <= 100000 ? 4 : 24;
+}
+// A launch takes at most this many, so that no kernel holds the GPU for long.
+constexpr int RESIDENT_MAX = 4096;
 
 struct ResidentPlan {
     std::vector<ResidentTile> tiles;  // one per CTA
     int w = 0, h = 0, gx = 0;
+    int min_steps = 0;                // resident_min of all nodes
     int threads = 0;
     size_t smem = 0;
     int device = 0, precision = 0;
@@ -54,6 +64,8 @@ struct Geo {
 
 constexpr size_t RESIDENT_SMEM = 220 * 1024;  // of 227 KB, beside the static part
 constexpr int RIM_NODES = 2;   // rim nodes a thread receives at most
+// Threads of the CTAs of tiles with more than 256 nodes.
+constexpr int resident_threads(bool f64) { return f64 ? 384 : 512; }
 
 // Cut the lattices (of one precision) so that every tile has an SM of its
 // own and fits its shared memory.  false when they are too large, too many,

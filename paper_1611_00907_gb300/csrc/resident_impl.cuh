@@ -12,7 +12,7 @@
 // that every SM gets one rectangle, of any size, and a step costs the
 // arithmetic of that rectangle plus one trip through L2.  Measured per step,
 // tile kernels (default shape, 16-step graphs) -> here: FP32 64 x 64 20.9 ->
-// 1.8 us, 256 x 128 6.7 -> 2.7, 512 x 512 7.5 -> 5.2, 704 x 704 9.6 -> 8.2;
+// 1.7 us, 256 x 128 6.7 -> 2.7, 512 x 512 7.5 -> 5.2, 704 x 704 9.6 -> 8.2;
 // FP64 64 x 64 47 -> 5.6 us, 256 x 256 39 -> 21, 500 x 200 40 -> 28, 512 x 512
 // 74 -> 64.  What bounds it: up to some 30 000 nodes the exchange and the
 // barriers (about 1.5 us), beyond that FP64 the FP64 units, FP32 issue.
@@ -109,36 +109,40 @@ template <> struct Word<double> {
 #endif
 
 // ---------------------------------------------------------------------------
-// A thread's nodes of one column, (x, y) .. (x, y + N - 1).  FP32: two, on
-// packed pairs with the functions of the two-nodes-per-lane path.  FP64: one,
-// since an FP64 instruction holds the SM quarter's FP64 unit for the same
-// time however few lanes are active, so on small tiles it is the number of
-// instructions per thread that counts.  i: index of the lower node in a
-// field of row width W.
+// A thread's nodes of one column, (x, y) .. (x, y + N - 1), N one or two.
+// FP32 computes on packed pairs with the functions of the two-nodes-per-lane
+// path: two nodes per thread, or, on tiles of at most a node per thread, one
+// (the other half of each pair idle), which halves the chain of shared-memory
+// accesses that a step of a small tile waits for.  FP64: one, since an FP64
+// instruction holds the SM quarter's FP64 unit for the same time however few
+// lanes are active, so on small tiles it is the number of instructions per
+// thread that counts.  i: index of the lower node in a field of row width W.
 // ---------------------------------------------------------------------------
-template <class real> constexpr int column_nodes() { return sizeof(real) == 8 ? 1 : 2; }
 struct Rows2 {
     Row2 d, m, u;
 };
+template <int N>
 __device__ __forceinline__ Rows2 rows2(const float *s, int i, int W)
 {
     Row<float> r[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) r[j] = row_of(s, i + (j - 1) * W);
+    for (int j = 0; j < 2 + N; ++j) r[j] = row_of(s, i + (j - 1) * W);
+    if (N == 1) r[3] = r[2];
     auto two = [&](int a) {
         return Row2{make_float2(r[a].c, r[a + 1].c), make_float2(r[a].h, r[a + 1].h),
                     make_float2(r[a].d, r[a + 1].d)};
     };
     return {two(0), two(1), two(2)};
 }
+template <int N>
 __device__ __forceinline__ void column_mu(const Consts<float> &K, float ref, const float *R,
-                                          int i, int W, float (&mu)[2])
+                                          int i, int W, float (&mu)[N])
 {
-    const Rows2 r = rows2(R, i, W);
+    const Rows2 r = rows2<N>(R, i, W);
     const float2 m = pfma(p2(-K.kappa), lap2(r.u, r.m, r.d),
                           mu_bulk2(K.eos, padd(r.m.c, p2(ref))));
     mu[0] = m.x;
-    mu[1] = m.y;
+    if constexpr (N == 2) mu[1] = m.y;
 }
 __device__ __forceinline__ void column_mu(const Consts<double> &K, double ref, const double *R,
                                           int i, int W, double (&mu)[1])
@@ -146,11 +150,12 @@ __device__ __forceinline__ void column_mu(const Consts<double> &K, double ref, c
     mu[0] = mu_of(K, R[i] + ref,
                   lap6(row_of(R, i + W), row_of(R, i), row_of(R, i - W)));
 }
+template <int N>
 __device__ __forceinline__ void column_collide(const Consts<float> &K, float ref, const float *R,
                                                int i, int W, const float *M, int j, int MW,
-                                               const float (&f)[2][9], float (&fp)[2][9])
+                                               const float (&f)[N][9], float (&fp)[N][9])
 {
-    const Rows2 r = rows2(R, i, W), m = rows2(M, j, MW);
+    const Rows2 r = rows2<N>(R, i, W), m = rows2<N>(M, j, MW);
     float2 grx, gry, gmx, gmy, g[9], gp[9];
     grad2(r.u, r.m, r.d, grx, gry);
     grad2(m.u, m.m, m.d, gmx, gmy);
@@ -158,12 +163,12 @@ __device__ __forceinline__ void column_collide(const Consts<float> &K, float ref
     const float2 Fx = psub(pmul(grx, third), pmul(rho, gmx));
     const float2 Fy = psub(pmul(gry, third), pmul(rho, gmy));
 #pragma unroll
-    for (int k = 1; k < 9; ++k) g[k] = make_float2(f[0][k], f[1][k]);
+    for (int k = 1; k < 9; ++k) g[k] = make_float2(f[0][k], f[N - 1][k]);
     collide2(g, drho, rho, Fx, Fy, p2(K.tau), p2(K.omega), gp);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         fp[0][k] = gp[k].x;
-        fp[1][k] = gp[k].y;
+        if constexpr (N == 2) fp[1][k] = gp[k].y;
     }
 }
 __device__ __forceinline__ void column_collide(const Consts<double> &K, double ref,
@@ -221,14 +226,14 @@ struct RimNode {
 };
 
 // WALLS: the variant of lattices with walls (batches: of any lattice).
-template <class S, int NT, bool BATCH, bool WALLS>
+template <class S, int NT, int N, bool BATCH, bool WALLS>
 __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResidentArgs A)
 {
     using real = typename S::real;
     using pop_t = typename S::pop_t;
     using rho_t = typename S::rho_t;
     using WD = Word<real>;
-    constexpr int N = column_nodes<real>();
+    static_assert(N == 1 || sizeof(real) == 4, "FP64: one node per thread");
     static_assert(sizeof(pop_t) == sizeof(real) && sizeof(rho_t) == sizeof(real),
                   "populations kept as stored");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -488,18 +493,21 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResidentArgs A)
     }
 }
 
-// Launch of one precision: threads 256 or 512 (ResidentPlan::threads).
+// Launch of one precision: threads 256, or RESIDENT_THREADS with two FP32
+// nodes per thread (ResidentPlan::threads).
 template <class S>
 cudaError_t launch_resident_t(const ResidentArgs &a, bool batch, int grid, int threads,
                               size_t smem, cudaStream_t s)
 {
-    void *const kern[2][3] = {{(void *)resident_kernel<S, 256, false, false>,
-                               (void *)resident_kernel<S, 256, false, true>,
-                               (void *)resident_kernel<S, 256, true, true>},
-                              {(void *)resident_kernel<S, 512, false, false>,
-                               (void *)resident_kernel<S, 512, false, true>,
-                               (void *)resident_kernel<S, 512, true, true>}};
-    void *k = kern[threads == 512][batch ? 2 : a.L.walls ? 1 : 0];
+    constexpr int NT = resident_threads(sizeof(typename S::real) == 8),
+                  N = sizeof(typename S::real) == 8 ? 1 : 2;
+    void *const kern[2][3] = {{(void *)resident_kernel<S, 256, 1, false, false>,
+                               (void *)resident_kernel<S, 256, 1, false, true>,
+                               (void *)resident_kernel<S, 256, 1, true, true>},
+                              {(void *)resident_kernel<S, NT, N, false, false>,
+                               (void *)resident_kernel<S, NT, N, false, true>,
+                               (void *)resident_kernel<S, NT, N, true, true>}};
+    void *k = kern[threads == NT][batch ? 2 : a.L.walls ? 1 : 0];
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)RESIDENT_SMEM);
     if (e != cudaSuccess) return e;
