@@ -374,6 +374,24 @@ lbm_status ensure_graph(lbm_batch *b)
     return LBM_OK;
 }
 
+// The shape a batch starts with (lbm_batch_autotune picks among all of them).
+// FP32 storage, every lattice three or more whole 64 x 32 tiles in each
+// direction (walls: the top row may be ragged, from four rows on): 64 x 32, two
+// nodes per lane; 32 walled lattices of 512 x 256 take 57.6 us a step on it, 63.7 on
+// 32 x 32.  Otherwise 32 x 32, whose path takes ragged last tiles: 32 uneven
+// lattices with sides of 64 to 1024 take 107.9 us, 124 on 64 x 32.
+void default_shape(const lbm_instance *inst, int count, int precision, int *tx, int *ty)
+{
+    bool wide = precision == LBM_F32 || precision == LBM_F32_OFFSET;
+    for (int i = 0; i < count && wide; ++i) {
+        const int rows = inst[i].walls ? inst[i].ny - 2 : inst[i].ny, left = rows % 32;
+        wide = inst[i].nx % 64 == 0 && inst[i].nx >= 192 && rows >= 96 &&
+               (inst[i].walls ? left == 0 || left >= 4 : left == 0);
+    }
+    *tx = wide ? 64 : 32;
+    *ty = 32;
+}
+
 lbm_status check_index(lbm_batch *b, int index)
 {
     if (index < 0 || index >= (int)b->inst.size())
@@ -426,9 +444,7 @@ lbm_status lbm_batch_create(const lbm_instance *inst, int count, int precision,
         }
         b->own_stream = true;
     }
-    // the default shape (lbm_batch_autotune picks among all of them)
-    b->tx = 32;
-    b->ty = 32;
+    default_shape(inst, count, precision, &b->tx, &b->ty);
     for (int i = 0; i < count && st == LBM_OK; ++i) {
         const lbm_instance &q = inst[i];
         lbm_config cfg{q.nx, q.ny, q.walls, q.tau, q.kappa, q.rho_ref, precision,
@@ -610,6 +626,7 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
     int sx[16], sy[16];
     const int n = step_shapes(sx, sy, 16);
     const long long t0 = b->t;
+    const int tx_stay = b->tx, ty_stay = b->ty;
     std::vector<long long> tsave;  // inactive lattices may lag the batch
     for (lbm_ctx *c : b->inst) tsave.push_back(c->t);
     int best = -1;
@@ -621,12 +638,12 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
     // configurations: every tile shape with a grid row per lattice (groups of
     // one geometry) or 1, 2 or 4 work items per CTA
     const int per[4] = {0, 1, 2, 4};
-    // and last (k == 4 n) the resident steps, on the default shape
+    // and last (k == 4 n) the resident steps, on the shape as it is
     auto restore = [&](int k) -> lbm_status {
         const bool stay = k == 4 * n;
         b->tiles_chosen = !stay;
-        b->tx = stay ? 32 : sx[k / 4];
-        b->ty = stay ? 32 : sy[k / 4];
+        b->tx = stay ? tx_stay : sx[k / 4];
+        b->ty = stay ? ty_stay : sy[k / 4];
         b->per_cta = stay ? 0 : per[k % 4];
         lbm_status s2 = rebuild(b);
         for (size_t i = 0; i < b->inst.size() && s2 == LBM_OK; ++i)
