@@ -506,6 +506,12 @@ __device__ void load_rho_tile(const Lattice &L, int cur, int X0, int Y0,
     using real = typename S::real;
     constexpr int W = TX + 4, H = TY + 4;
     const int wx = min(TX, L.nx - X0), wy = min(TY, L.nyf - Y0);
+    // a halo that touches no edge of the lattice needs no wrap and no wall rule
+    if (X0 >= 2 && X0 + TX + 2 <= L.nx && Y0 >= 2 && Y0 + TY + 2 <= L.nyf) {
+        for (int k = threadIdx.x; k < W * H; k += blockDim.x)
+            s_rho[k] = load_rho_stored<S>(L, cur, Y0 + k / W - 2, X0 + k % W - 2);
+        return;
+    }
     for (int k = threadIdx.x; k < W * H; k += blockDim.x) {
         const int lx = k % W, ly = k / W;
         if (lx > wx + 3 || ly > wy + 3) {  // beyond a ragged tile's halo

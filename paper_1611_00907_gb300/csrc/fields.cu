@@ -15,7 +15,7 @@ namespace cplbm {
 // directions share the even part of Eq. 14 and the factors are applied once,
 // 35 FP64 instructions a node against 60 for the eight expressions written
 // out.  It leaves the snapshot of the reductions behind as well, which took a
-// pass of macro_kernel.  1500 x 1100 FP64: 203 + 320 -> 110 us.
+// pass of macro_kernel.  1500 x 1100 FP64: 203 + 320 -> 135 us.
 // A block takes 64 x 4 nodes.
 // ---------------------------------------------------------------------------
 constexpr int INIT_X = 64, INIT_Y = 4;
@@ -23,7 +23,7 @@ constexpr int INIT_X = 64, INIT_Y = 4;
 template <class S>
 __global__ void __launch_bounds__(INIT_X *INIT_Y)
     init_kernel(const Lattice L, const double *rho_in, const double *ux_in,
-                const double *uy_in, double *prev, int *bad, int blocks_x)
+                const double *uy_in, double *prev, int *bad, int blocks_x, double pole)
 {
     using pop_t = typename S::pop_t;
     using rho_t = typename S::rho_t;
@@ -34,7 +34,6 @@ __global__ void __launch_bounds__(INIT_X *INIT_Y)
     const long long g = (long long)(r + L.walls) * L.nx + x;  // lattice index
     const double rho = rho_in[g];
     const double ux = ux_in ? ux_in[g] : 0.0, uy = uy_in ? uy_in[g] : 0.0;
-    const double pole = (L.eos.kind == EOS_CS ? 4.0 : 1.0) / L.eos.b;
     if (!(rho > 0.0 && rho < pole && isfinite(ux) && isfinite(uy)))
         atomicAdd(bad, 1);
     const double ref = S::offset ? L.rho_ref : 0.0;
@@ -84,6 +83,22 @@ __device__ __forceinline__ void atomic_max_nonneg(double *addr, double v)
     atomicMax((unsigned long long *)addr, (unsigned long long)__double_as_longlong(v));
 }
 
+// A population: no store of the kernel touches it, so the loads of a thread's
+// rows need not wait for the stores of the rows before (with them in order the
+// reductions waited for memory eight times in a row: 2048 x 2048 FP32 314 us).
+__device__ __forceinline__ double ld_stable(const double *p) { return __ldg(p); }
+__device__ __forceinline__ float ld_stable(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float ld_stable(const __half *p) { return __half2float(__ldg(p)); }
+// Tests and comparisons of doubles on their bits: the FP64 units do the
+// floating-point ones.  Non-negative doubles order like their bits.
+__device__ __forceinline__ bool finite64(double v)
+{
+    return ((unsigned)__double2hiint(v) & 0x7FF00000u) != 0x7FF00000u;
+}
+__device__ __forceinline__ unsigned long long magnitude(double v)
+{
+    return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+}
 // FP64 values of FP32 results without the FP64 units, which do the type
 // conversions too (widen): subnormal values count as zero.
 __device__ __forceinline__ double to_f64(double v) { return v; }
@@ -129,13 +144,16 @@ __device__ __forceinline__ void half_force(const Consts<double> &, const double 
     py = (1.0 / 72.0) * gry + (r * gmy + jy);
 }
 
-// Bound by the FP64 units, in FP64 (67 FP64 instructions a node) and, with
-// velocities or reductions, in FP32 too (the division and the sums are FP64
-// in every storage).  1500 x 1100 FP64: 367 -> 190 us for the four fields.
+// FP64 is bound by the FP64 units (about 70 FP64 instructions a node): 1500 x
+// 1100, the four fields 367 -> 250 us; FP32 by instruction issue and latency
+// (the division and the sums are FP64 in every storage): 4096 x 4096, density
+// and velocity 829 -> 413 us with four blocks of 64 registers per SM (476 with
+// three), the sums 847 -> 433.
 template <class S, int TX, int TY>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sizeof(typename S::real) == 8 ? 3 : 4)
     macro_kernel(const Lattice L, int parity, int cur, double *o_rho, double *o_vx,
-                 double *o_vy, double *o_mu, double *red, double *prev, int *bad)
+                 double *o_vy, double *o_mu, double *red, double *prev, int *bad,
+                 long long tiles, int tiles_x)
 {
     using real = typename S::real;
     using pop_t = typename S::pop_t;
@@ -145,119 +163,159 @@ __global__ void __launch_bounds__(256)
     extern __shared__ unsigned char smem_raw[];
     real *s_rho = reinterpret_cast<real *>(smem_raw);
     real *s_mu = s_rho + (TY + 4) * WR;
-    __shared__ double s_red[4][32];
+    __shared__ double s_sum[4][256];
     __shared__ int s_bad;
 
-    const int X0 = blockIdx.x * TX, Y0 = blockIdx.y * TY;
-    const int wx = min(TX, L.nx - X0), wy = min(TY, L.nyf - Y0);
     if (threadIdx.x == 0) s_bad = 0;
-    load_rho_tile<S, TX, TY>(L, cur, X0, Y0, s_rho);
-    __syncthreads();
-    mu_tile<S, TX, TY>(L, X0, Y0, s_rho, s_mu);
-    __syncthreads();
-
+    const bool flow = o_vx || o_vy || red;   // otherwise no population is needed
     const Consts<real> &K = consts<real>(L);
     const real rho_ref = S::offset ? K.rho_ref : real(0);
     const pop_t *A = (const pop_t *)L.pops;
-    const bool flow = o_vx || o_vy || red;   // otherwise no population is needed
-    double acc_m = 0.0, acc_x = 0.0, acc_y = 0.0, acc_d = 0.0;
-    // s_rho holds the stored form; rho_ref makes it absolute
+    double acc_m = 0.0, acc_x = 0.0, acc_y = 0.0;
+    unsigned long long acc_d = 0;  // magnitude of a non-negative double
     int nbad = 0;
-    const int lx = threadIdx.x % TX, ly0 = threadIdx.x / TX * PER;
-    const int cr0 = (ly0 + 1) * WR + lx + 2, cm0 = ly0 * WM + lx + 1;
-    Row<real> rd = row_of(s_rho, cr0), rm = row_of(s_rho, cr0 + WR);
-    Row<real> md = row_of(s_mu, cm0), mm = row_of(s_mu, cm0 + WM);
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int X0 = (int)(tile % tiles_x) * TX, Y0 = (int)(tile / tiles_x) * TY;
+        const int wx = min(TX, L.nx - X0), wy = min(TY, L.nyf - Y0);
+        load_rho_tile<S, TX, TY>(L, cur, X0, Y0, s_rho);
+        __syncthreads();
+        if (flow || o_mu) {  // otherwise the density is all that is asked for
+            mu_tile<S, TX, TY>(L, X0, Y0, s_rho, s_mu);
+            __syncthreads();
+        }
+
+        // Tiles away from the lattice's edges read each direction at a constant
+        // offset; the general addressing took a third of the instructions.
+        const bool inside = X0 >= 1 && X0 + TX < L.nx && Y0 >= 1 && Y0 + TY < L.nyf;
+        long long off[9];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int ly = ly0 + k;
-        const Row<real> ru = row_of(s_rho, cr0 + (k + 2) * WR);
-        const Row<real> mu = row_of(s_mu, cm0 + (k + 2) * WM);
-        if (lx < wx && ly < wy) {
-            const int x = X0 + lx, r = Y0 + ly;
-            const long long g = (long long)(r + L.walls) * L.nx + x;
-            const real rho = rm.c + rho_ref;
-            const double rho64 = to_f64(rho);
-            if (o_rho) o_rho[g] = rho64;
-            if (o_mu) o_mu[g] = to_f64(mm.c);
-            if (flow) {
-                real f[9];
+        for (int i = 1; i < 9; ++i)
+            off[i] = parity == 0 ? (i - 1) * L.plane
+                                 : (opp(i) - 1) * L.plane - (long long)ey(i) * L.pitch - ex(i);
+        // the snapshot's rows ahead of the work that needs them
+        double before[PER];
+        if (red && prev) {
 #pragma unroll
-                for (int i = 1; i < 9; ++i) {
-                    const pop_t *p = A + aa_read_index(L, parity, i, r, x);
-                    f[i] = CPLBM_IN_POPS(L, p, 1) ? ld_real(p) : real(0);
-                }
-                real grx, gry, gmx, gmy;
-                grad12(ru, rm, rd, grx, gry);
-                grad12(mu, mm, md, gmx, gmy);
-                double px, py;  // rho v
-                half_force(K, f, rho, grx, gry, gmx, gmy, px, py);
-                const double ir = inverse(rho64);
-                if (o_vx) o_vx[g] = px * ir;
-                if (o_vy) o_vy[g] = py * ir;
-                if (red) {
-                    acc_m += rho64;
-                    acc_x += px;
-                    acc_y += py;
-                    if (!(isfinite(rho64) && isfinite(px) && isfinite(py))) ++nbad;
-                    if (prev) {
-                        const double d = fabs(rho64 - prev[g]);
-                        acc_d = fmax(acc_d, isfinite(d) ? d : 0.0);
-                        prev[g] = rho64;
+            for (int k = 0; k < PER; ++k) {
+                const int x = threadIdx.x % TX, y = threadIdx.x / TX * PER + k;
+                before[k] = x < wx && y < wy
+                                ? prev[(long long)(Y0 + y + L.walls) * L.nx + X0 + x] : 0.0;
+            }
+        }
+        // s_rho holds the stored form; rho_ref makes it absolute
+        const int lx = threadIdx.x % TX, ly0 = threadIdx.x / TX * PER;
+        const int cr0 = (ly0 + 1) * WR + lx + 2, cm0 = ly0 * WM + lx + 1;
+        Row<real> rd = row_of(s_rho, cr0), rm = row_of(s_rho, cr0 + WR);
+        Row<real> md = row_of(s_mu, cm0), mm = row_of(s_mu, cm0 + WM);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int ly = ly0 + k;
+            const Row<real> ru = row_of(s_rho, cr0 + (k + 2) * WR);
+            const Row<real> mu = row_of(s_mu, cm0 + (k + 2) * WM);
+            if (lx < wx && ly < wy) {
+                const int x = X0 + lx, r = Y0 + ly;
+                const long long g = (long long)(r + L.walls) * L.nx + x;
+                const real rho = rm.c + rho_ref;
+                const double rho64 = to_f64(rho);
+                if (o_rho) o_rho[g] = rho64;
+                if (o_mu) o_mu[g] = to_f64(mm.c);
+                if (flow) {
+                    real f[9];
+                    if (inside) {
+                        const pop_t *q = A + fidx(L, r, x);
+#pragma unroll
+                        for (int i = 1; i < 9; ++i)
+                            f[i] = CPLBM_IN_POPS(L, q + off[i], 1) ? ld_stable(q + off[i]) : real(0);
+                    } else {
+#pragma unroll
+                        for (int i = 1; i < 9; ++i) {
+                            const pop_t *p = A + aa_read_index(L, parity, i, r, x);
+                            f[i] = CPLBM_IN_POPS(L, p, 1) ? ld_stable(p) : real(0);
+                        }
+                    }
+                    real grx, gry, gmx, gmy;
+                    grad12(ru, rm, rd, grx, gry);
+                    grad12(mu, mm, md, gmx, gmy);
+                    double px, py;  // rho v
+                    half_force(K, f, rho, grx, gry, gmx, gmy, px, py);
+                    if (o_vx || o_vy) {
+                        const double ir = inverse(rho64);
+                        if (o_vx) o_vx[g] = px * ir;
+                        if (o_vy) o_vy[g] = py * ir;
+                    }
+                    if (red) {
+                        acc_m += rho64;
+                        acc_x += px;
+                        acc_y += py;
+                        if (!(finite64(rho64) && finite64(px) && finite64(py))) ++nbad;
+                        if (prev) {
+                            const double d = rho64 - before[k];
+                            if (finite64(d)) acc_d = max(acc_d, magnitude(d));
+                            prev[g] = rho64;
+                        }
                     }
                 }
             }
+            rd = rm;
+            rm = ru;
+            md = mm;
+            mm = mu;
         }
-        rd = rm;
-        rm = ru;
-        md = mm;
-        mm = mu;
-    }
-    // Solid rows: rho by Eq. 28 and the wall mu from the shared tiles.
-    if (L.walls && (o_rho || o_mu || o_vx || o_vy)) {
-        for (int lx = threadIdx.x; lx < wx; lx += blockDim.x) {
-            const int x = X0 + lx;
-            if (Y0 == 0) {
-                const long long g = x;
-                if (o_rho) o_rho[g] = (double)(s_rho[1 * WR + lx + 2] + rho_ref);
-                if (o_mu) o_mu[g] = (double)s_mu[0 * WM + lx + 1];
-                if (o_vx) o_vx[g] = 0.0;
-                if (o_vy) o_vy[g] = 0.0;
-            }
-            if (Y0 + wy == L.nyf) {
-                const long long g = (long long)(L.ny - 1) * L.nx + x;
-                if (o_rho) o_rho[g] = (double)(s_rho[(wy + 2) * WR + lx + 2] + rho_ref);
-                if (o_mu) o_mu[g] = (double)s_mu[(wy + 1) * WM + lx + 1];
-                if (o_vx) o_vx[g] = 0.0;
-                if (o_vy) o_vy[g] = 0.0;
+        // Solid rows: rho by Eq. 28 and the wall mu from the shared tiles.
+        if (L.walls && (o_rho || o_mu || o_vx || o_vy)) {
+            for (int lx = threadIdx.x; lx < wx; lx += blockDim.x) {
+                const int x = X0 + lx;
+                if (Y0 == 0) {
+                    const long long g = x;
+                    if (o_rho) o_rho[g] = (double)(s_rho[1 * WR + lx + 2] + rho_ref);
+                    if (o_mu) o_mu[g] = (double)s_mu[0 * WM + lx + 1];
+                    if (o_vx) o_vx[g] = 0.0;
+                    if (o_vy) o_vy[g] = 0.0;
+                }
+                if (Y0 + wy == L.nyf) {
+                    const long long g = (long long)(L.ny - 1) * L.nx + x;
+                    if (o_rho) o_rho[g] = (double)(s_rho[(wy + 2) * WR + lx + 2] + rho_ref);
+                    if (o_mu) o_mu[g] = (double)s_mu[(wy + 1) * WM + lx + 1];
+                    if (o_vx) o_vx[g] = 0.0;
+                    if (o_vy) o_vy[g] = 0.0;
+                }
             }
         }
+        __syncthreads();  // the next tile reuses the shared memory
     }
     if (red) {
-        // warp then block reduction, fixed order within the block
-        for (int o = 16; o > 0; o >>= 1) {
-            acc_m += __shfl_down_sync(0xffffffffu, acc_m, o);
-            acc_x += __shfl_down_sync(0xffffffffu, acc_x, o);
-            acc_y += __shfl_down_sync(0xffffffffu, acc_y, o);
-            acc_d = fmax(acc_d, __shfl_down_sync(0xffffffffu, acc_d, o));
-        }
-        const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+        // block reduction in a fixed order: the threads' sums by columns of
+        // eight in the first warp, then across its lanes (FP64 additions on
+        // one warp of the block instead of all eight)
         if (nbad) atomicAdd(&s_bad, nbad);
-        if (lane == 0) {
-            s_red[0][warp] = acc_m; s_red[1][warp] = acc_x;
-            s_red[2][warp] = acc_y; s_red[3][warp] = acc_d;
-        }
+        s_sum[0][threadIdx.x] = acc_m;
+        s_sum[1][threadIdx.x] = acc_x;
+        s_sum[2][threadIdx.x] = acc_y;
+        s_sum[3][threadIdx.x] = __longlong_as_double((long long)acc_d);
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (threadIdx.x < 32) {
             double m = 0, sx = 0, sy = 0, d = 0;
-            for (int w = 0; w < (int)(blockDim.x / 32); ++w) {
-                m += s_red[0][w]; sx += s_red[1][w]; sy += s_red[2][w];
-                d = fmax(d, s_red[3][w]);
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                const int t = threadIdx.x + 32 * w;
+                m += s_sum[0][t];
+                sx += s_sum[1][t];
+                sy += s_sum[2][t];
+                d = fmax(d, s_sum[3][t]);
             }
-            atomicAdd(&red[0], m);
-            atomicAdd(&red[1], sx);
-            atomicAdd(&red[2], sy);
-            atomic_max_nonneg(&red[3], d);
-            if (s_bad) atomicAdd(bad, s_bad);
+            for (int o = 16; o > 0; o >>= 1) {
+                m += __shfl_down_sync(0xffffffffu, m, o);
+                sx += __shfl_down_sync(0xffffffffu, sx, o);
+                sy += __shfl_down_sync(0xffffffffu, sy, o);
+                d = fmax(d, __shfl_down_sync(0xffffffffu, d, o));
+            }
+            if (threadIdx.x == 0) {
+                atomicAdd(&red[0], m);
+                atomicAdd(&red[1], sx);
+                atomicAdd(&red[2], sy);
+                atomic_max_nonneg(&red[3], d);
+                if (s_bad) atomicAdd(bad, s_bad);
+            }
         }
     }
 }
@@ -313,10 +371,14 @@ static cudaError_t launch_init_t(const Lattice &L, const double *rho,
                                  int *bad, cudaStream_t s)
 {
     const int bx = (L.nx + INIT_X - 1) / INIT_X, by = (L.nyf + INIT_Y - 1) / INIT_Y;
+    const double pole = (L.eos.kind == EOS_CS ? 4.0 : 1.0) / L.eos.b;
     init_kernel<S><<<(unsigned)bx * (unsigned)by, INIT_X * INIT_Y, 0, s>>>(L, rho, ux, uy, prev,
-                                                                          bad, bx);
+                                                                          bad, bx, pole);
     return cudaGetLastError();
 }
+
+// Four rounds of three blocks on each of 152 SMs.
+constexpr long long MACRO_SUM_BLOCKS = 152 * 3 * 4;
 
 template <class S, int TY>
 static cudaError_t launch_macro_ty(const Lattice &L, int parity, int cur, double *rho,
@@ -326,9 +388,13 @@ static cudaError_t launch_macro_ty(const Lattice &L, int parity, int cur, double
     using real = typename S::real;
     constexpr int TX = FIELD_TILE_X;
     const size_t smem = sizeof(real) * ((TY + 4) * (TX + 4) + (TY + 2) * (TX + 2));
-    dim3 grid((L.nx + TX - 1) / TX, (L.nyf + TY - 1) / TY);
+    const int tiles_x = (L.nx + TX - 1) / TX;
+    const long long tiles = (long long)tiles_x * ((L.nyf + TY - 1) / TY);
+    // The sums end in four atomics per block on the same four words: a bounded
+    // number of blocks, each with several tiles of a large lattice.
+    const unsigned grid = (unsigned)(red ? std::min(tiles, MACRO_SUM_BLOCKS) : tiles);
     macro_kernel<S, TX, TY><<<grid, 256, smem, s>>>(L, parity, cur, rho, vx, vy, mu, red, prev,
-                                                    bad);
+                                                    bad, tiles, tiles_x);
     return cudaGetLastError();
 }
 
