@@ -148,8 +148,13 @@ lbm_status plan_resident(lbm_batch *b, std::vector<Lattice> &lats)
 // Steps queued as resident launches (0 when they do not apply).
 int resident_steps(lbm_batch *b, int left)
 {
+    if (b->plan.tiles.empty() || left < b->plan.min_steps) return 0;
+    // a caller's capture takes plain launches, as for one lattice
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+        return 0;
     int done = 0;
-    while (!b->plan.tiles.empty() && left - done >= b->plan.min_steps) {
+    while (left - done >= b->plan.min_steps) {
         const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
         if (launch_resident(b->plan, nullptr, b->d_lats, b->d_tiles, n, (int)(b->t & 1),
                             b->xchg_tag, b->stream) != cudaSuccess) {

@@ -363,4 +363,8 @@ bool host_critical(int kind, double a, double b, double R, double *Tc,
 double host_alpha(int kind, double Tr, double omega);
 void set_global_error(const char *msg);
 
+// noalloc.cu: the unique ID of the current CUDA context (a device reset makes
+// a new one); false where the driver cannot tell.
+bool current_context_id(unsigned long long *id);
+
 }  // namespace cplbm

@@ -104,12 +104,12 @@ cudaError_t launch_prec(int prec, const ResidentArgs &a, bool batch, int grid, i
 
 // Resident launches of one device follow one another whatever streams they
 // are on: two of them, each holding a part of the SMs, would wait for the
-// rest.  One event per device, kept for the life of the process.
+// rest.  One event per device and CUDA context: a device reset ends both.
 constexpr int MAX_DEVICES = 64;
 struct Turn {
     std::mutex m;
     cudaEvent_t done = nullptr;
-    cudaStream_t last = nullptr;
+    unsigned long long ctx_id = 0;
 };
 Turn g_turn[MAX_DEVICES];
 
@@ -196,14 +196,24 @@ cudaError_t launch_resident(const ResidentPlan &p, const Lattice *single, const 
     a.tag = tag;
     Turn &t = g_turn[p.device];
     std::lock_guard<std::mutex> lock(t.m);
-    cudaError_t e = cudaSuccess;
-    if (!t.done) e = cudaEventCreateWithFlags(&t.done, cudaEventDisableTiming);
-    else if (t.last != s) e = cudaStreamWaitEvent(s, t.done, 0);
-    if (e != cudaSuccess) return e;
+    unsigned long long id = 0;
+    current_context_id(&id);
+    if (!t.done || t.ctx_id != id) {
+        t.done = nullptr;
+        cudaError_t e = cudaEventCreateWithFlags(&t.done, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            t.done = nullptr;
+            return e;
+        }
+        t.ctx_id = id;
+    } else {  // on the launch's own stream too: a stream's handle may be used again
+        cudaError_t e = cudaStreamWaitEvent(s, t.done, 0);
+        if (e != cudaSuccess) return e;
+    }
     const int grid = (int)p.tiles.size();
-    e = launch_prec(p.precision, a, single == nullptr, grid, p.threads, p.smem, s);
-    if (e == cudaSuccess) e = cudaEventRecord(t.done, s);
-    t.last = s;
+    cudaError_t e = launch_prec(p.precision, a, single == nullptr, grid, p.threads, p.smem, s);
+    // unrecorded, the event would let the next launch overlap this one
+    if (e == cudaSuccess && cudaEventRecord(t.done, s) != cudaSuccess) e = cudaStreamSynchronize(s);
     return e;
 }
 

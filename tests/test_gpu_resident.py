@@ -115,6 +115,33 @@ def test_batch_of_small_lattices_fp64(oracle_threads):
                 assert _rel(got[key], want[key]) < 1e-12, (k, key)
 
 
+def test_batch_steps_inside_a_callers_graph_capture(oracle_threads):
+    """A block of batch steps that the caller captures into its own CUDA graph
+    is launched on the tile kernels and may be replayed: a resident launch
+    could not, the tags of its exchange words are those of one run."""
+    import torch
+    sim, ref = _sim("cs", 70, 21, False, "f64", 1.1)
+    sim.close()
+    _, par, rho, ux, uy, mc = _state("cs", 70, 21, False)
+    stream = torch.cuda.Stream()
+    with Batch([dict(nx=70, ny=21, eos="cs", a=par[0], b=par[1], Tr=0.85, tau=1.1, kappa=par[2],
+                     mu_bottom=mc + 0.01)], precision="f64", stream=stream.cuda_stream) as b:
+        b.init(0, rho, ux, uy)
+        b.step(2)                         # kernel attributes set outside the capture
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            b.step(8)
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        b.step(4)                         # resident, from where the replays ended
+        ref.step(2 + 3 * 8 + 4)
+        got, want = b.moments(0), ref.moments()
+        for key in ("rho", "mu", "vx", "vy"):
+            assert _rel(got[key], want[key]) < 1e-12, key
+
+
 def test_wait_limit_leaves_the_state_and_is_reported():
     # a limit of zero cycles: every tile gives up at its first exchange
     lib = _lib.load()
