@@ -216,7 +216,7 @@ bool pt_shape_supported(int prec, int tx, int ty);
 // edge has the layout of an interior halo.  That ragged last tile takes the
 // TMA path too with bit 3, its right and top edges at the tile's own width
 // and height: on 32-wide tiles always, on 64-wide ones in the single-lattice
-// kernels with the ragged variant (ragged_seam; batches keep such tiles on the
+// FP32 kernels with the ragged variant (ragged_seam; batches keep such tiles on the
 // general path or, by default, take 32-wide tiles: an uneven batch of 32
 // lattices, sides 64 to 1024, ran at 108 us a step on 32 x 32, 122 on 64 x 16
 // with ragged tiles on the TMA path).  Walls: at least

@@ -1969,17 +1969,19 @@ static cudaError_t launch_shape(const Lattice &L, int parity, int cur,
     // Tile classes (tile_kind): the TMA paths also take the seam tiles of
     // periodic edges.  A lattice whose sides are no multiples of a 64-wide
     // tile takes the kernel whose edge tiles may be ragged, unless what is
-    // left over is too narrow for it (seam_bits); 1001 x 757 FP32 offset: 25.0
-    // -> 16.4 us a step against those tiles on the general path.
+    // left over is too narrow for it (seam_bits); 1001 x 757 FP32 offset: 26.0
+    // -> 16.4 us a step against those tiles on the general path.  FP32 storage
+    // only: the two paths round in different order, which flips stored halves,
+    // and over 150 steps a 224 x 96 FP16 lattice's velocities then differed by
+    // 1.2 % from those of the general path.
     const int ntx = (L.nx + TX - 1) / TX, nty = (L.nyf + TY - 1) / TY;
     const int rx = L.nx % TX, ry = L.nyf % TY;
     int seams = HasTma<S, TX, TY, NT>::value || HasTmaPair<S, TX, TY, NT>::value
                     ? seam_bits(L, TX, TY) : 0;
-    const bool rag = HasTmaPair<S, TX, TY, NT>::value && m.valid &&
-                     ragged_seam(L, TX, TY, seams);
+    constexpr bool R = HasTmaPair<S, TX, TY, NT>::value && sizeof(typename S::pop_t) == 4;
+    const bool rag = R && m.valid && ragged_seam(L, TX, TY, seams);
     if (rag) seams |= 8;
-    // kernels by ragged last tiles, walls and parity
-    constexpr bool R = HasTmaPair<S, TX, TY, NT>::value;  // others: one kernel for both
+    // kernels by ragged last tiles (without R one kernel for both), walls and parity
     void (*const kern[2][2][2])(const Lattice, int, int, const TmaMaps) = {
         {{step_kernel<S, TX, TY, NT, 0, false, false>, step_kernel<S, TX, TY, NT, 1, false, false>},
          {step_kernel<S, TX, TY, NT, 0, true, false>, step_kernel<S, TX, TY, NT, 1, true, false>}},
