@@ -150,14 +150,16 @@ lbm_status lbm_init(lbm_ctx *ctx, const double *rho, const double *ux,
 /* Queue nsteps (>= 0) time steps (Sec. II: density, Eq. 8, Eq. 12, the
  * BGK collision of Eq. 13-14 and streaming, with the wall rule of Sec. IV)
  * on the context's stream.  Returns without waiting for the GPU.  Four steps
- * or more (24 in FP32 storage above 100 000 nodes) of a lattice whose state fits the shared memory of all SMs together
- * (FP64 up to about 270 000 nodes, FP32 storage about 500 000; not FP16, the
- * pressure-tensor force or a chosen tile shape) run as one cooperative launch
- * that keeps the state there; such launches follow one another on a device.
- * Otherwise blocks of 16 steps replay a CUDA graph captured on a private stream at the first
- * such call (and again after any change of tile shape, physics, force
- * model or wait limit); while the context's stream is being captured by
- * the caller, every step is a plain launch that joins the caller's graph. */
+ * or more (24 in FP32 storage above 100 000 nodes) of a lattice whose state
+ * fits the shared memory of all SMs together (FP64 up to about 270 000 nodes,
+ * FP32 storage with walls, or once lbm_autotune has found it faster, about
+ * 500 000; not FP16, the pressure-tensor force or a chosen tile shape) run as
+ * one cooperative launch that keeps the state there; such launches follow one
+ * another on a device.  Otherwise blocks of 16 steps replay a CUDA graph
+ * captured on a private stream at the first such call (and again after any
+ * change of tile shape, physics, force model or wait limit); while the
+ * context's stream is being captured by the caller, every step is a plain
+ * launch that joins the caller's graph. */
 lbm_status lbm_step(lbm_ctx *ctx, int nsteps);
 
 /* Macroscopic fields of the current state: rho (solid rows: Eq. 28), the
@@ -247,8 +249,7 @@ lbm_status lbm_batch_reduce(lbm_batch *b, int index, double out[4]);
 /* Tile shape of the batched kernel (as lbm_set_tile; default 32x32, or 64x32
  * in FP32 storage when 64x32 tiles fit every lattice and at least three stand
  * side by side, a ragged top row of four or more below a wall allowed), or
- * the fastest configuration measured over nsteps steps (every tile shape
- * with each schedule of lbm_batch_schedule: 0 when some group of lattices
+ * the fastest configuration measured over nsteps steps (every tile shape with each schedule of lbm_batch_schedule: 0 when some group of lattices
  * qualifies, 1, 2 and 4) with the state restored afterwards; *tx, *ty
  * receive the shape kept. */
 lbm_status lbm_batch_set_tile(lbm_batch *b, int tx, int ty);

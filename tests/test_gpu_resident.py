@@ -78,11 +78,15 @@ def test_blocks_of_steps_fp64(size, walls, blocks, oracle_threads):
 @pytest.mark.parametrize("walls", [False, True])
 def test_blocks_of_steps_fp32_match_the_tile_kernels(precision, walls):
     for size in SIZES[3:]:
-        sim, _ = _sim("cs", *size, walls, precision, 1.0)
         tiles, _ = _sim("cs", *size, walls, precision, 1.0)
-        with sim, tiles:
+        _, par, rho, ux, uy, mc = _state("cs", *size, walls)
+        spec = dict(nx=size[0], ny=size[1], eos="cs", a=par[0], b=par[1], Tr=0.85, omega=0.344,
+                    tau=1.0, kappa=par[2], walls=walls, mu_bottom=mc + 0.01, mu_top=mc - 0.01)
+        # (a batch: a periodic FP32 lattice by itself stays on the tile kernels)
+        with Batch([spec], precision=precision) as many, tiles:
+            many.init(0, rho, ux, uy)
             tiles.set_tile(64, 16)
-            a, b = sim.step(30).moments(), tiles.step(30).moments()
+            a, b = many.step(30).moments(0), tiles.step(30).moments()
             drho = 3.6e-6 * b["rho"].max()
             for key, tol in (("rho", drho), ("mu", 6 * drho), ("vx", 12 * drho),
                              ("vy", 12 * drho)):
