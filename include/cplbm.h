@@ -246,10 +246,11 @@ lbm_status lbm_batch_moments(lbm_batch *b, int index, double *rho, double *vx,
 lbm_status lbm_batch_populations(lbm_batch *b, int index, double *f,
                                  int on_device);
 lbm_status lbm_batch_reduce(lbm_batch *b, int index, double out[4]);
-/* Tile shape of the batched kernel (as lbm_set_tile; default 32x32, or 64x32
+/* Tile shape of the batched kernel (as lbm_set_tile; default 32x32; 64x32
  * in FP32 storage when 64x32 tiles fit every lattice and at least three stand
- * side by side, a ragged top row of four or more below a wall allowed), or
- * the fastest configuration measured over nsteps steps (every tile shape with each schedule of lbm_batch_schedule: 0 when some group of lattices
+ * side by side, a ragged top row of four or more below a wall allowed; 32x16
+ * in FP64 below 2 000 000 nodes in all), or the fastest configuration
+ * measured over nsteps steps (every tile shape with each schedule of lbm_batch_schedule: 0 when some group of lattices
  * qualifies, 1, 2 and 4) with the state restored afterwards; *tx, *ty
  * receive the shape kept. */
 lbm_status lbm_batch_set_tile(lbm_batch *b, int tx, int ty);

@@ -384,9 +384,15 @@ lbm_status ensure_graph(lbm_batch *b)
 // direction (walls: the top row may be ragged, from four rows on): 64 x 32, two
 // nodes per lane; 32 walled lattices of 512 x 256 take 57.6 us a step on it, 63.7 on
 // 32 x 32.  Otherwise 32 x 32, whose path takes ragged last tiles: 32 uneven
-// lattices with sides of 64 to 1024 take 107.9 us, 124 on 64 x 32.
+// lattices with sides of 64 to 1024 take 107.9 us, 124 on 64 x 32.  FP64, which
+// the arithmetic of the fullest SM bounds, below some thirteen 32 x 32 tiles
+// per SM: 32 x 16, whose finer tiles spread more evenly (16 uneven lattices up
+// to 400 a side 217 -> 200 us, 6 walled ones of 228 x 105 76 -> 61; 1024 x 1024
+// alone 250 -> 260, its halo costs more).
 void default_shape(const lbm_instance *inst, int count, int precision, int *tx, int *ty)
 {
+    long long nodes = 0;
+    for (int i = 0; i < count; ++i) nodes += (long long)inst[i].nx * inst[i].ny;
     bool wide = precision == LBM_F32 || precision == LBM_F32_OFFSET;
     for (int i = 0; i < count && wide; ++i) {
         const int rows = inst[i].walls ? inst[i].ny - 2 : inst[i].ny, left = rows % 32;
@@ -394,7 +400,7 @@ void default_shape(const lbm_instance *inst, int count, int precision, int *tx, 
                (inst[i].walls ? left == 0 || left >= 4 : left == 0);
     }
     *tx = wide ? 64 : 32;
-    *ty = 32;
+    *ty = precision == LBM_F64 && nodes < 2000000 ? 16 : 32;
 }
 
 lbm_status check_index(lbm_batch *b, int index)
