@@ -231,7 +231,9 @@ lbm_status lbm_batch_init(lbm_batch *b, int index, const double *rho,
 /* Queue nsteps steps of every active lattice; all must be initialised.  Four
  * steps or more (24, as for lbm_step) of lattices that together fit the shared memory of all SMs
  * run on the chip, as lbm_step's (not after lbm_batch_set_tile or
- * lbm_batch_schedule with a schedule). */
+ * lbm_batch_schedule with a schedule); the batch takes the memory of the words
+ * their tiles exchange at the first such call, and steps as other batches do
+ * where it is not to be had. */
 lbm_status lbm_batch_step(lbm_batch *b, int nsteps);
 /* Take lattice `index` out of the batched launch (active = 0) or put it
  * back (active = 1).  An inactive lattice keeps its state and step count and

@@ -64,9 +64,11 @@ struct lbm_batch {
     // (resident.cu), unless the caller has chosen a tile shape or schedule
     bool tiles_chosen = false;
     ResidentPlan plan;             // of the active lattices; empty: none
-    ResidentTile *d_tiles = nullptr;
+    std::vector<Lattice> on;       // their descriptors, tiles' inst counts them
+    bool staged = false;           // both are on the device, with exchange words:
+    char *d_stage = nullptr;       // descriptors, then tiles
     void *d_xchg = nullptr;
-    size_t xchg_cap = 0;
+    size_t stage_cap = 0, xchg_cap = 0;
     unsigned xchg_tag = 1;
     std::string err;
 };
@@ -103,46 +105,68 @@ void drop_graph(lbm_batch *b)
 }
 
 // Cut the active lattices for the resident steps, when all of them together
-// fit the GPU's shared memory: their tiles, and the exchange words that
-// their descriptors (copies in lats) point to.
-lbm_status plan_resident(lbm_batch *b, std::vector<Lattice> &lats)
+// fit the GPU's shared memory.
+void plan_resident(lbm_batch *b, const std::vector<Lattice> &lats)
 {
-    std::vector<Lattice> on;
-    std::vector<int> index;
+    b->on.clear();
     for (size_t i = 0; i < lats.size(); ++i)
-        if (b->active[i]) {
-            on.push_back(lats[i]);
-            index.push_back((int)i);
-        }
+        if (b->active[i]) b->on.push_back(lats[i]);
     ResidentPlan p;
-    if (on.empty() || !resident_plan(on.data(), (int)on.size(), b->device, &p)) return LBM_OK;
-    size_t need = 0;
-    for (const Lattice &L : on) need += xchg_bytes(L);
-    if (need > b->xchg_cap) {
-        dev_free(b->d_xchg);
-        b->d_xchg = nullptr;
-        b->xchg_cap = 0;
-        BCUDA(b, dev_alloc(&b->d_xchg, need));
-        b->xchg_cap = need;
-        // zero is no step's tag; words of an earlier cut carry older tags
-        BCUDA(b, cudaMemsetAsync(b->d_xchg, 0, need, b->stream));
-    }
+    if (!b->on.empty() && resident_plan(b->on.data(), (int)b->on.size(), b->device, &p))
+        b->plan = std::move(p);
+}
+
+// The plan's tiles, descriptors and exchange words, at the first resident
+// launch after the plan was made: a batch that makes none does not hold them,
+// and one that cannot have them steps on the tile kernels (false), as a
+// lattice by itself.  (Another stream of this thread may be capturing.)
+bool stage_resident(lbm_batch *b)
+{
+    if (b->staged) return true;
+    size_t words = 0;
+    for (const Lattice &L : b->on) words += xchg_bytes(L);
+    const size_t lats = b->on.size() * sizeof(Lattice),
+                 bytes = lats + b->plan.tiles.size() * sizeof(ResidentTile);
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+    auto grow = [](void **p, size_t *cap, size_t need) {
+        if (need <= *cap) return cudaSuccess;
+        dev_free(*p);
+        *cap = 0;
+        cudaError_t e = dev_alloc(p, need);
+        if (e == cudaSuccess) *cap = need;
+        return e;
+    };
+    const size_t had = b->xchg_cap;
+    cudaError_t e = grow(&b->d_xchg, &b->xchg_cap, words);
+    // zero is no step's tag; words of an earlier cut carry older tags
+    if (e == cudaSuccess && b->xchg_cap != had)
+        e = cudaMemsetAsync(b->d_xchg, 0, words, b->stream);
+    if (e == cudaSuccess) e = grow((void **)&b->d_stage, &b->stage_cap, bytes);
     char *x = (char *)b->d_xchg;
-    for (int i : index) {
-        lats[i].xchg = x;
+    for (Lattice &L : b->on) {
+        L.xchg = x;
 #ifdef CPLBM_CHECK_BOUNDS
-        lats[i].b_xchg = (long long)xchg_bytes(lats[i]);
+        L.b_xchg = (long long)xchg_bytes(L);
 #endif
-        x += xchg_bytes(lats[i]);
+        x += xchg_bytes(L);
     }
-    for (ResidentTile &t : p.tiles) t.inst = index[t.inst];
-    dev_free(b->d_tiles);
-    b->d_tiles = nullptr;
-    BCUDA(b, dev_alloc((void **)&b->d_tiles, p.tiles.size() * sizeof(ResidentTile)));
-    BCUDA(b, cudaMemcpy(b->d_tiles, p.tiles.data(), p.tiles.size() * sizeof(ResidentTile),
-                        cudaMemcpyHostToDevice));
-    b->plan = std::move(p);
-    return LBM_OK;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_stage, b->on.data(), lats, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_stage + lats, b->plan.tiles.data(), bytes - lats,
+                            cudaMemcpyHostToDevice, b->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        dev_free(b->d_xchg);
+        dev_free(b->d_stage);
+        b->d_xchg = nullptr;
+        b->d_stage = nullptr;
+        b->xchg_cap = b->stage_cap = 0;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    b->staged = e == cudaSuccess;
+    return b->staged;
 }
 
 // Steps queued as resident launches (0 when they do not apply).
@@ -153,11 +177,17 @@ int resident_steps(lbm_batch *b, int left)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
         return 0;
+    if (!stage_resident(b)) {
+        b->plan = ResidentPlan{};
+        return 0;
+    }
+    const Lattice *d_on = reinterpret_cast<const Lattice *>(b->d_stage);
+    const ResidentTile *d_tiles = reinterpret_cast<const ResidentTile *>(d_on + b->on.size());
     int done = 0;
     while (left - done >= b->plan.min_steps) {
         const int n = left - done < RESIDENT_MAX ? left - done : RESIDENT_MAX;
-        if (launch_resident(b->plan, nullptr, b->d_lats, b->d_tiles, n, (int)(b->t & 1),
-                            b->xchg_tag, b->stream) != cudaSuccess) {
+        if (launch_resident(b->plan, nullptr, d_on, d_tiles, n, (int)(b->t & 1), b->xchg_tag,
+                            b->stream) != cudaSuccess) {
             cudaGetLastError();  // no co-resident launch here: the tile kernels
             b->plan = ResidentPlan{};
             break;
@@ -175,6 +205,7 @@ lbm_status rebuild(lbm_batch *b)
 {
     drop_graph(b);
     b->plan = ResidentPlan{};
+    b->staged = false;
     const int n = (int)b->inst.size();
     std::vector<Lattice> lats;
     std::vector<WorkItem> items;
@@ -271,10 +302,7 @@ lbm_status rebuild(lbm_batch *b)
         }
         b->groups.push_back(std::move(grp));
     }
-    if (!b->tiles_chosen && b->inst[0]->use_tma) {
-        lbm_status st = plan_resident(b, lats);
-        if (st != LBM_OK) return st;
-    }
+    if (!b->tiles_chosen && b->inst[0]->use_tma) plan_resident(b, lats);
     dev_free(b->d_lats);
     dev_free(b->d_items);
     b->d_lats = nullptr;
@@ -726,7 +754,7 @@ void lbm_batch_destroy(lbm_batch *b)
     for (lbm_ctx *c : b->inst) lbm_destroy(c);
     dev_free(b->d_lats);
     dev_free(b->d_items);
-    dev_free(b->d_tiles);
+    dev_free(b->d_stage);
     dev_free(b->d_xchg);
     for (cudaStream_t st : b->aux) cudaStreamDestroy(st);
     for (cudaEvent_t ev : b->joins) cudaEventDestroy(ev);
