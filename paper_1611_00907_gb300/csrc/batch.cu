@@ -104,18 +104,6 @@ void drop_graph(lbm_batch *b)
     b->exec = nullptr;
 }
 
-// Cut the active lattices for the resident steps, when all of them together
-// fit the GPU's shared memory.
-void plan_resident(lbm_batch *b, const std::vector<Lattice> &lats)
-{
-    b->on.clear();
-    for (size_t i = 0; i < lats.size(); ++i)
-        if (b->active[i]) b->on.push_back(lats[i]);
-    ResidentPlan p;
-    if (!b->on.empty() && resident_plan(b->on.data(), (int)b->on.size(), b->device, &p))
-        b->plan = std::move(p);
-}
-
 // The plan's tiles, descriptors and exchange words, at the first resident
 // launch after the plan was made: a batch that makes none does not hold them,
 // and one that cannot have them steps on the tile kernels (false), as a
@@ -199,21 +187,43 @@ int resident_steps(lbm_batch *b, int left)
     return done;
 }
 
-// Apply the batch tile shape to every lattice and rebuild the device copies
-// of the descriptors, the work list and the groups' tensor maps.
-lbm_status rebuild(lbm_batch *b)
+// What the launches of one choice of active lattices and tile shape are made
+// of: device copies of the descriptors and the work list, and the groups.
+struct Launches {
+    std::vector<char> active;
+    int tx = 0, ty = 0;
+    std::vector<Group> groups;
+    std::vector<Lattice> on;   // active ones
+    ResidentPlan plan;         // their cut for the resident steps
+    Lattice *d_lats = nullptr;
+    WorkItem *d_items = nullptr;
+    int n_items = 0;
+    Launches() = default;
+    Launches(const Launches &) = delete;
+    ~Launches()
+    {
+        dev_free(d_lats);
+        dev_free(d_items);
+    }
+};
+
+// Make them, leaving the batch and its lattices as they are: a failure leaves
+// what steps the batch now in place.  stay: cut the active lattices for the
+// resident steps too, if all of them together fit the GPU's shared memory.
+lbm_status build_launches(lbm_batch *b, std::vector<char> active, int tx, int ty, bool stay,
+                          Launches &f)
 {
-    drop_graph(b);
-    b->plan = ResidentPlan{};
-    b->staged = false;
     const int n = (int)b->inst.size();
+    f.active = std::move(active);
+    f.tx = tx;
+    f.ty = ty;
     std::vector<Lattice> lats;
     std::vector<WorkItem> items;
+    std::vector<TmaMaps> maps(BATCH_LAUNCH_LATTICES);  // of the group's lattices
     // edge tiles (periodic seams, wall rows) take the TMA paths too: the
     // 32-wide one, and for FP32 arithmetic the 64-wide pair path
     // (step_batch_kernel); FP64 64-wide tiles have no TMA path
-    const bool tma_shape = b->tx == 32 || (b->tx == 64 && b->precision != LBM_F64);
-    b->groups.clear();
+    const bool tma_shape = tx == 32 || (tx == 64 && b->precision != LBM_F64);
     for (int g0 = 0; g0 < n; g0 += BATCH_LAUNCH_LATTICES) {
         Group grp;
         grp.inst0 = g0;
@@ -225,25 +235,26 @@ lbm_status rebuild(lbm_batch *b)
         }
         std::vector<WorkItem> gen, edge, inner;
         for (int i = g0; i < n && i < g0 + BATCH_LAUNCH_LATTICES; ++i) {
-            lbm_ctx *c = b->inst[i];
-            c->L.tx = b->tx;
-            c->L.ty = b->ty;
-            ctx_refresh_maps(c);
+            const lbm_ctx *c = b->inst[i];
             lats.push_back(c->L);
-            const bool maps_ok = tma_shape && c->use_tma && c->maps.valid;
+            Lattice &L = lats.back();
+            L.tx = tx;
+            L.ty = ty;
+            TmaMaps &m = maps[i - g0];
+            ctx_maps(c, L, &m);
+            const bool maps_ok = tma_shape && m.valid;
             if (maps_ok)
                 for (int p = 0; p < 2; ++p) {
-                    grp.maps[p]->pops[i - g0] = c->maps.pops;
-                    grp.maps[p]->rho[i - g0] = c->maps.rho[p];
+                    grp.maps[p]->pops[i - g0] = m.pops;
+                    grp.maps[p]->rho[i - g0] = m.rho[p];
                 }
-            if (!b->active[i]) continue;
-            const Lattice &L = c->L;
-            const int ntx = (L.nx + b->tx - 1) / b->tx, nty = (L.nyf + b->ty - 1) / b->ty;
-            const int seams = tma_shape ? seam_bits(L, b->tx, b->ty) : 0;
+            if (!f.active[i]) continue;
+            const int ntx = (L.nx + tx - 1) / tx, nty = (L.nyf + ty - 1) / ty;
+            const int seams = tma_shape ? seam_bits(L, tx, ty) : 0;
             const int no_tma = maps_ok ? 0 : ITEM_NO_TMA;
             for (int by = 0; by < nty; ++by)
                 for (int bx = 0; bx < ntx; ++bx) {
-                    const int kind = tile_kind(L, b->tx, b->ty, bx, by, seams);
+                    const int kind = tile_kind(L, tx, ty, bx, by, seams);
                     (kind == TILE_GENERAL ? gen : kind == TILE_SEAM ? edge : inner)
                         .push_back({i, bx, by, kind | no_tma});
                 }
@@ -270,17 +281,17 @@ lbm_status rebuild(lbm_batch *b)
         int first = -1;
         bool same = grp.tma_only && grp.n_items > 0;
         for (int i = g0; same && i < n && i < g0 + BATCH_LAUNCH_LATTICES; ++i) {
-            if (!b->active[i]) continue;
-            const Lattice &L = b->inst[i]->L;
+            if (!f.active[i]) continue;
+            const Lattice &L = lats[i];
             if (first < 0) first = i;
-            const Lattice &F = b->inst[first]->L;
+            const Lattice &F = lats[first];
             same = L.nx == F.nx && L.ny == F.ny && L.walls == F.walls;
         }
         if (same && first >= 0) {
-            const Lattice &F = b->inst[first]->L;
-            grp.ntx = (F.nx + b->tx - 1) / b->tx;
-            grp.nty = (F.nyf + b->ty - 1) / b->ty;
-            grp.seams = seam_bits(F, b->tx, b->ty);
+            const Lattice &F = lats[first];
+            grp.ntx = (F.nx + tx - 1) / tx;
+            grp.nty = (F.nyf + ty - 1) / ty;
+            grp.seams = seam_bits(F, tx, ty);
             grp.walls = F.walls != 0;
             for (int p = 0; p < 2; ++p) {
                 grp.uniform[p].reset(new (std::nothrow) UniformGroup);
@@ -289,34 +300,33 @@ lbm_status rebuild(lbm_batch *b)
             }
             int k = 0;
             for (int i = g0; i < n && i < g0 + BATCH_LAUNCH_LATTICES; ++i) {
-                if (!b->active[i]) continue;
-                const lbm_ctx *c = b->inst[i];
+                if (!f.active[i]) continue;
                 for (int p = 0; p < 2; ++p) {
-                    grp.uniform[p]->pops[k] = c->maps.pops;
-                    grp.uniform[p]->rho[k] = c->maps.rho[p];
-                    grp.uniform[p]->L[k] = c->L;
+                    grp.uniform[p]->pops[k] = maps[i - g0].pops;
+                    grp.uniform[p]->rho[k] = maps[i - g0].rho[p];
+                    grp.uniform[p]->L[k] = lats[i];
                 }
                 ++k;
             }
             grp.n_uniform = k;
         }
-        b->groups.push_back(std::move(grp));
+        f.groups.push_back(std::move(grp));
     }
-    if (!b->tiles_chosen && b->inst[0]->use_tma) plan_resident(b, lats);
-    dev_free(b->d_lats);
-    dev_free(b->d_items);
-    b->d_lats = nullptr;
-    b->d_items = nullptr;
-    BCUDA(b, dev_alloc((void **)&b->d_lats, lats.size() * sizeof(Lattice)));
-    BCUDA(b, dev_alloc((void **)&b->d_items, (items.size() + 1) * sizeof(WorkItem)));
-    BCUDA(b, cudaMemcpy(b->d_lats, lats.data(), lats.size() * sizeof(Lattice),
+    if (stay && b->inst[0]->use_tma) {
+        for (int i = 0; i < n; ++i)
+            if (f.active[i]) f.on.push_back(lats[i]);
+        if (!f.on.empty()) resident_plan(f.on.data(), (int)f.on.size(), b->device, &f.plan);
+    }
+    BCUDA(b, dev_alloc((void **)&f.d_lats, lats.size() * sizeof(Lattice)));
+    BCUDA(b, dev_alloc((void **)&f.d_items, (items.size() + 1) * sizeof(WorkItem)));
+    BCUDA(b, cudaMemcpy(f.d_lats, lats.data(), lats.size() * sizeof(Lattice),
                         cudaMemcpyHostToDevice));
     if (!items.empty())
-        BCUDA(b, cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(WorkItem),
+        BCUDA(b, cudaMemcpy(f.d_items, items.data(), items.size() * sizeof(WorkItem),
                             cudaMemcpyHostToDevice));
-    b->n_items = (int)items.size();
+    f.n_items = (int)items.size();
     // one stream and join event per group after the first, for the graph
-    while (b->aux.size() + 1 < b->groups.size()) {
+    while (b->aux.size() + 1 < f.groups.size()) {
         cudaStream_t st = nullptr;
         cudaEvent_t ev = nullptr;
         BCUDA(b, cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
@@ -324,9 +334,30 @@ lbm_status rebuild(lbm_batch *b)
         BCUDA(b, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
         b->joins.push_back(ev);
     }
-    if (!b->fork && b->groups.size() > 1)
+    if (!b->fork && f.groups.size() > 1)
         BCUDA(b, cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
     return LBM_OK;
+}
+
+// Put them in the place of the batch's present ones.
+void use_launches(lbm_batch *b, Launches &f)
+{
+    drop_graph(b);
+    for (lbm_ctx *c : b->inst) {
+        c->L.tx = f.tx;
+        c->L.ty = f.ty;
+        ctx_refresh_maps(c);
+    }
+    b->tx = f.tx;
+    b->ty = f.ty;
+    b->active.swap(f.active);
+    b->groups.swap(f.groups);
+    std::swap(b->d_lats, f.d_lats);
+    std::swap(b->d_items, f.d_items);
+    b->n_items = f.n_items;
+    b->on.swap(f.on);
+    std::swap(b->plan, f.plan);
+    b->staged = false;
 }
 
 BatchList work_list(const lbm_batch *b, const Group &g, int cur)
@@ -501,7 +532,11 @@ lbm_status lbm_batch_create(const lbm_instance *inst, int count, int precision,
         if (st != LBM_OK) bfail(b, st, "lattice %d: %s", i, lbm_last_error(c));
         b->nodes += (long long)q.nx * q.ny;
     }
-    if (st == LBM_OK) st = rebuild(b);
+    if (st == LBM_OK) {
+        Launches f;
+        st = build_launches(b, b->active, b->tx, b->ty, true, f);
+        if (st == LBM_OK) use_launches(b, f);
+    }
     if (st != LBM_OK) {
         g_batch_err = b->err;
         lbm_batch_destroy(b);
@@ -574,9 +609,13 @@ lbm_status lbm_batch_set_active(lbm_batch *b, int index, int active)
                      "only after an even number of batch steps (now %lld)", b->t);
     const char want = active ? 1 : 0;
     if (b->active[index] == want) return LBM_OK;
-    b->active[index] = want;
     BCUDA(b, cudaSetDevice(b->device));
-    return rebuild(b);
+    std::vector<char> on = b->active;
+    on[index] = want;
+    Launches f;
+    st = build_launches(b, std::move(on), b->tx, b->ty, !b->tiles_chosen, f);
+    if (st == LBM_OK) use_launches(b, f);
+    return st;
 }
 
 lbm_status lbm_batch_moments(lbm_batch *b, int index, double *rho, double *vx,
@@ -616,15 +655,15 @@ lbm_status lbm_batch_set_tile(lbm_batch *b, int tx, int ty)
     if (!step_shape_supported(b->precision, tx, ty))
         return bfail(b, LBM_ERR_ARG, "no step kernel for tile %d x %d", tx, ty);
     BCUDA(b, cudaSetDevice(b->device));
+    Launches f;
+    lbm_status st = build_launches(b, b->active, tx, ty, false, f);
     // re-split each lattice's current density for the new tile grid
-    for (lbm_ctx *c : b->inst) {
-        lbm_status st = forward(b, c, lbm_set_tile(c, tx, ty));
-        if (st != LBM_OK) return st;
-    }
-    b->tx = tx;
-    b->ty = ty;
+    for (size_t i = 0; i < b->inst.size() && st == LBM_OK; ++i)
+        st = forward(b, b->inst[i], lbm_set_tile(b->inst[i], tx, ty));
+    if (st != LBM_OK) return st;
     b->tiles_chosen = true;
-    return rebuild(b);
+    use_launches(b, f);
+    return LBM_OK;
 }
 
 lbm_status lbm_batch_schedule(lbm_batch *b, int items_per_cta, int *current)
@@ -665,7 +704,8 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
     int sx[16], sy[16];
     const int n = step_shapes(sx, sy, 16);
     const long long t0 = b->t;
-    const int tx_stay = b->tx, ty_stay = b->ty;
+    const int tx_stay = b->tx, ty_stay = b->ty, per_cta = b->per_cta;
+    const bool tiles_chosen = b->tiles_chosen, saved = st == LBM_OK;
     std::vector<long long> tsave;  // inactive lattices may lag the batch
     for (lbm_ctx *c : b->inst) tsave.push_back(c->t);
     int best = -1;
@@ -678,18 +718,26 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
     // one geometry) or 1, 2 or 4 work items per CTA
     const int per[4] = {0, 1, 2, 4};
     // and last (k == 4 n) the resident steps, on the shape as it is
+    auto state_back = [&]() -> lbm_status {  // as a whole, for any tile shape
+        lbm_status s2 = LBM_OK;
+        b->t = t0;
+        for (size_t i = 0; i < b->inst.size(); ++i) {
+            b->inst[i]->t = tsave[i];
+            const lbm_status s3 = ctx_snapshot(b->inst[i], snaps[i], false);
+            if (s3 != LBM_OK) s2 = s3;
+        }
+        return s2;
+    };
     auto restore = [&](int k) -> lbm_status {
         const bool stay = k == 4 * n;
+        Launches f;
+        lbm_status s2 = build_launches(b, b->active, stay ? tx_stay : sx[k / 4],
+                                       stay ? ty_stay : sy[k / 4], stay, f);
+        if (s2 != LBM_OK) return s2;
         b->tiles_chosen = !stay;
-        b->tx = stay ? tx_stay : sx[k / 4];
-        b->ty = stay ? ty_stay : sy[k / 4];
         b->per_cta = stay ? 0 : per[k % 4];
-        lbm_status s2 = rebuild(b);
-        for (size_t i = 0; i < b->inst.size() && s2 == LBM_OK; ++i)
-            s2 = ctx_snapshot(b->inst[i], snaps[i], false);
-        b->t = t0;
-        for (size_t i = 0; i < b->inst.size(); ++i) b->inst[i]->t = tsave[i];
-        return s2;
+        use_launches(b, f);
+        return state_back();
     };
     for (int k = 0; k <= 4 * n && st == LBM_OK; ++k) {
         if (k < 4 * n && !step_shape_supported(b->precision, sx[k / 4], sy[k / 4])) continue;
@@ -724,6 +772,18 @@ lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty)
         st = restore(best);
         if (st == LBM_OK && cudaStreamSynchronize(b->stream) != cudaSuccess)
             st = bfail(b, LBM_ERR_CUDA, "synchronize");
+    }
+    if (st != LBM_OK && saved) {  // as it was, as far as that goes
+        const std::string err = b->err;
+        Launches f;
+        b->tiles_chosen = tiles_chosen;
+        b->per_cta = per_cta;
+        if (build_launches(b, b->active, tx_stay, ty_stay, !tiles_chosen, f) == LBM_OK)
+            use_launches(b, f);
+        else
+            drop_graph(b);  // the captured launches carry another grid
+        state_back();
+        b->err = err;
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);

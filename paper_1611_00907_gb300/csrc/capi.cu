@@ -255,12 +255,7 @@ void free_all(lbm_ctx *c)
 
 // Tensor maps for the current tile shape (the TMA path is skipped when they
 // cannot be built, e.g. for FP16 storage).
-void refresh_maps(lbm_ctx *c)
-{
-    char msg[256];
-    c->maps.valid = 0;
-    if (c->use_tma) build_tma_maps(c->L, &c->maps, msg, sizeof msg);
-}
+void refresh_maps(lbm_ctx *c) { ctx_maps(c, c->L, &c->maps); }
 
 lbm_status report_flags(lbm_ctx *c, int flags)
 {
@@ -1112,4 +1107,10 @@ lbm_status ctx_snapshot(lbm_ctx *c, char *snap, bool save)
     return snapshot(c, snap, save);
 }
 void ctx_refresh_maps(lbm_ctx *c) { refresh_maps(c); }
+void ctx_maps(const lbm_ctx *c, const Lattice &L, TmaMaps *m)
+{
+    char msg[256];
+    m->valid = 0;
+    if (c->use_tma) build_tma_maps(L, m, msg, sizeof msg);
+}
 }  // namespace cplbm

@@ -59,4 +59,6 @@ lbm_status ctx_snapshot(lbm_ctx *c, char *snap, bool save);
 lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out);
 // capi.cu: rebuild the TMA maps after a tile-shape change.
 void ctx_refresh_maps(lbm_ctx *c);
+// ... and the maps of its buffers for the tile shape of L.
+void ctx_maps(const lbm_ctx *c, const Lattice &L, TmaMaps *m);
 }  // namespace cplbm

@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 from oracle import thermo
-from paper_1611_00907_gb300 import Batch, Simulation, _lib, inputs
+from paper_1611_00907_gb300 import Batch, LbmError, Simulation, _lib, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -83,4 +83,61 @@ def test_steps_without_the_on_chip_steps_memory(failing, oracle_threads):
         held = lib.lbm_test_device_allocs()
         b.step(16)
         assert lib.lbm_test_device_allocs() == held + 2
+        _compare(b, refs)
+
+
+def _fails(n, call):
+    lib = _lib.load()
+    lib.lbm_test_fail_device_alloc(n)
+    with pytest.raises(LbmError) as ei:
+        call()
+    lib.lbm_test_fail_device_alloc(-1)
+    assert ei.value.status == _lib.LBM_ERR_OOM
+
+
+@pytest.mark.parametrize("tile", [None, (32, 32)])
+@pytest.mark.parametrize("failing", [0, 1])
+def test_a_failed_change_leaves_the_batch_as_it_was(failing, tile, oracle_threads):
+    """A change of the active lattices or of the tile shape that runs out of
+    memory changes nothing: the batch goes on with the lattices, shape and work
+    list it had."""
+    specs, rhos, refs = _lattices()
+    with _batch(specs, rhos) as b:
+        if tile:
+            b.set_tile(*tile)
+        was = b.info()["tile"]
+        b.step(4)
+        _fails(failing, lambda: b.set_active(0, False))
+        b.step(18)                              # every lattice still moves
+        _fails(failing, lambda: b.set_tile(64, 16))
+        assert b.info()["tile"] == was
+        b.step(18)
+        for ref in refs:
+            ref.step(40)
+        _compare(b, refs)
+        b.set_active(1, False).step(18)
+        _fails(failing, lambda: b.set_active(1, True))
+        b.step(18)                              # the middle one still rests
+        for k in (0, 2):
+            refs[k].step(36)
+        _compare(b, refs)
+        b.set_active(1, True).step(18)
+        for ref in refs:
+            ref.step(18)
+        _compare(b, refs)
+
+
+@pytest.mark.parametrize("failing", range(9))
+def test_a_failed_autotune_leaves_the_batch_as_it_was(failing, oracle_threads):
+    """Its state copies (three lattices) or a candidate's work list cannot be
+    had: state, step counts and tile shape are those before the call."""
+    specs, rhos, refs = _lattices()
+    with _batch(specs, rhos) as b:
+        was = b.info()["tile"]
+        b.step(6)
+        _fails(failing, lambda: b.autotune(4))
+        assert b.info()["tile"] == was and b.info()["steps"] == 6
+        b.step(19)
+        for ref in refs:
+            ref.step(25)
         _compare(b, refs)
