@@ -500,7 +500,10 @@ lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
     for (int k = 0; k < 2 && st == LBM_OK; ++k)
         if (cudaMemsetAsync(L.rho[k], 0, (size_t)L.plane * rb, c->stream) != cudaSuccess)
             st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
-    if (st == LBM_OK && cudaMemset(c->d_report, 0, sizeof(Report)) != cudaSuccess)
+    // (on the context's stream: the default stream may reach it only after the
+    // context's first kernels have written there)
+    if (st == LBM_OK &&
+        cudaMemsetAsync(c->d_report, 0, sizeof(Report), c->stream) != cudaSuccess)
         st = fail(nullptr, LBM_ERR_CUDA, "cudaMemset failed");
     if (st != LBM_OK) {
         free_all(c);
