@@ -42,6 +42,10 @@ constexpr int MAX_CTAS = 152;   // one per SM; more samples take several rounds
 __host__ __device__ constexpr int layer_k(int l) { return l == 0 ? DIN : H; }
 __host__ __device__ constexpr int layer_n(int l) { return l == NL - 1 ? DOUT : H; }
 
+// Groups of SAMPLES samples.  (Counted in groups, the loops over them stay
+// within an int for every B.)
+__host__ __device__ constexpr int groups(int B) { return B / SAMPLES + (B % SAMPLES != 0); }
+
 // Offsets of layer l's weights [k][n] and biases in the flat parameter
 // arrays (FP32 masters, gradients, Adam moments share the layout).
 __host__ __device__ constexpr int w_off(int l)
@@ -289,7 +293,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     Biases Bs;
     load_weights<false>(P, W);
     load_biases(P, Bs);
-    for (int s0 = blockIdx.x * SAMPLES; s0 < B; s0 += gridDim.x * SAMPLES) {
+    for (int q = blockIdx.x; q < groups(B); q += gridDim.x) {
+        const int s0 = q * SAMPLES;
         forward(W, Bs, S, X, nin, B, s0);
         const int s = threadIdx.x / DOUT, c = threadIdx.x % DOUT;
         if (s0 + s < B && c < nout) Y[(long long)(s0 + s) * nout + c] = S.out[threadIdx.x];
@@ -361,7 +366,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     after_predecessor();
     load_weights<true>(P, W);
     load_biases(P, Bs);
-    for (int s0 = blockIdx.x * SAMPLES; s0 < B; s0 += gridDim.x * SAMPLES) {
+    for (int q = blockIdx.x; q < groups(B); q += gridDim.x) {
+        const int s0 = q * SAMPLES;
         forward(W, Bs, S, X, nin, B, s0);
         {   // output delta: d(mean sq error)/dy = 2 (y - t) / (B nout)
             const int s = threadIdx.x / DOUT, c = threadIdx.x % DOUT, gs = s0 + s;
@@ -470,7 +476,7 @@ lbm_status mfail(lbm_mlp *m, lbm_status s, const char *msg, cudaError_t e)
 
 Params params_of(const lbm_mlp *m) { return Params{m->wt, m->w, m->p}; }
 
-int ctas(int B) { return std::min((B + SAMPLES - 1) / SAMPLES, MAX_CTAS); }
+int ctas(int B) { return std::min(groups(B), MAX_CTAS); }
 
 // A launch that may start while its predecessor on the stream still runs
 // (the kernel waits for it, after_predecessor).

@@ -165,3 +165,22 @@ def test_gradient_matches_reference_elementwise():
         assert np.linalg.norm(got - ref) < norm_tol * np.linalg.norm(ref), k
         if k != 7:   # the output bias takes the unrounded delta in both models
             assert np.linalg.norm(got - plain[sl]) > norm_tol * np.linalg.norm(ref), k
+
+
+def test_prediction_of_almost_two_to_the_31_samples():
+    """The largest sample counts an int holds: the loop over groups of samples
+    ends inside it (17 GB of inputs and outputs)."""
+    import torch
+    B = 2 ** 31 - 1000
+    m = mlp.Mlp(seed=3)
+    X = torch.arange(B, dtype=torch.int32, device="cuda").remainder_(1021).to(torch.float32)
+    X.div_(1021.0)
+    X = X.view(B, 1)
+    Y = m.predict(X, 1)
+    for lo, hi in ((0, 4096), (B // 2, B // 2 + 4096), (B - 4096, B)):
+        lo -= lo % 16                    # the same groups of 16 samples
+        want = m.predict(X[lo:hi].contiguous(), 1)
+        assert torch.equal(Y[lo:hi], want), lo
+    del X, Y
+    torch.cuda.empty_cache()
+    m.close()
