@@ -42,8 +42,11 @@
 // which each of them published only after it had received all words of
 // step k (a block barrier stands between).  The launch is cooperative, so
 // all CTAs are resident and every wait ends; it is bounded all the same
-// (Lattice::wait_cycles), and a CTA that gives up raises ERR_WAIT_TIMEOUT and
-// leaves the lattice's global state as it was.
+// (Lattice::wait_cycles).  A CTA stores its part of the state, populations and
+// density, once it has received every rim of the call; one that gives up
+// raises ERR_WAIT_TIMEOUT and stores nothing.  Others may have finished by
+// then, and the host counts the steps of the call: a lattice whose time-out
+// has been reported is inconsistent until it is initialised or loaded again.
 #pragma once
 #include <type_traits>
 
@@ -413,14 +416,6 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResidentArgs A)
                     for (int i = 0; i < 9; ++i, q += L.plane)
                         if (CPLBM_IN_XCHG(L, q)) WD::put(q, fp[j][i], tag);
                 }
-                if (last) {
-                    pop_t *P = (pop_t *)L.pops;
-#pragma unroll
-                    for (int i = 1; i < 9; ++i) {
-                        pop_t *q = P + aa_write_index(L, (A.parity + k) & 1, i, y0 + yj, x0 + x);
-                        if (CPLBM_IN_POPS(L, q, 1)) *q = (pop_t)fp[j][i];
-                    }
-                }
             }
         }
 
@@ -455,6 +450,18 @@ __global__ void __launch_bounds__(NT, 1) resident_kernel(const ResidentArgs A)
             }
         }
         if (__syncthreads_or(!ok)) return false;
+        if (last) {  // every rim of the call is here: the populations back
+            pop_t *P = (pop_t *)L.pops;
+            for (int n = tid; n < w * h; n += NT) {
+                const int y = div_by(n, iw), x = n - y * w, c = cell(x, y);
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    pop_t *q = P + aa_write_index(L, (A.parity + k) & 1, i, y0 + y, x0 + x);
+                    if (CPLBM_IN_POPS(L, q, 1))
+                        *q = (pop_t)pull(kind, opp(i), c, first_row(y), last_row(y));
+                }
+            }
+        }
 
         // 5. The next density (tile-kernel order of the sum).
         constexpr int next = kind ^ 1;
