@@ -122,9 +122,10 @@ lbm_status lbm_get_tile(const lbm_ctx *ctx, int *tx, int *ty);
 /* Time nsteps (rounded up to an even count >= 2) steps of each compiled
  * tile shape of the force model in use (lbm_set_force_model) on the
  * context's own lattice, and of the on-chip steps of a small lattice
- * (lbm_step; *tx, *ty then receive the default shape), keep the fastest, and
- * restore
- * the state exactly as it was (the step counter included).  Allocates one
+ * (lbm_step; over 64 steps at least, loading and storing the state included;
+ * *tx, *ty then receive the default shape), keep the fastest per step, and
+ * restore the state exactly as it was (the step counter included; after an
+ * error the shape and the kind of step too).  Allocates one
  * temporary copy of the state.  *tx, *ty (may be NULL) receive the shape. */
 lbm_status lbm_autotune(lbm_ctx *ctx, int nsteps, int *tx, int *ty);
 
@@ -251,10 +252,12 @@ lbm_status lbm_batch_reduce(lbm_batch *b, int index, double out[4]);
 /* Tile shape of the batched kernel (as lbm_set_tile; default 32x32; 64x32
  * in FP32 storage when 64x32 tiles fit every lattice and at least three stand
  * side by side, a ragged top row of four or more below a wall allowed; 32x16
- * in FP64 below 2 000 000 nodes in all), or the fastest configuration
- * measured over nsteps steps (every tile shape with each schedule of lbm_batch_schedule: 0 when some group of lattices
- * qualifies, 1, 2 and 4) with the state restored afterwards; *tx, *ty
- * receive the shape kept. */
+ * in FP64 below 2 000 000 nodes in all), or the configuration that measures
+ * fastest per step: every tile shape with each schedule of lbm_batch_schedule
+ * (0 when some group of lattices qualifies, 1, 2 and 4) over nsteps steps,
+ * and the on-chip steps of a small batch over 64 at least (*tx, *ty then
+ * receive the shape the batch had).  The state is restored afterwards, after
+ * an error the configuration too; *tx, *ty receive the shape kept. */
 lbm_status lbm_batch_set_tile(lbm_batch *b, int tx, int ty);
 lbm_status lbm_batch_autotune(lbm_batch *b, int nsteps, int *tx, int *ty);
 /* Schedule of the batched kernel.  The lattices go to the GPU in groups of

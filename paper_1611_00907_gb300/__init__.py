@@ -185,8 +185,9 @@ class Simulation:
         return self
 
     def autotune(self, nsteps=20):
-        """Time every tile shape on this lattice, keep the fastest; the state
-        is left unchanged.  Returns the shape."""
+        """Time every tile shape on this lattice, and the on-chip steps of a
+        small one, and keep the fastest; the state is left unchanged.
+        Returns the shape."""
         tx, ty = C.c_int(), C.c_int()
         self._check(self._lib.lbm_autotune(self._ctx, int(nsteps), C.byref(tx),
                                            C.byref(ty)))

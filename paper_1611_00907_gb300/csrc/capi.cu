@@ -722,13 +722,16 @@ lbm_status lbm_autotune(lbm_ctx *c, int nsteps, int *best_tx, int *best_ty)
     int tx[16], ty[16];
     const int n = step_shapes(tx, ty, 16);
     const long long t0 = c->t;
+    const int tx0 = L.tx, ty0 = L.ty;
+    const bool resident0 = c->resident;
     int best = -1;
-    float best_ms = 0.f;
+    float best_us = 0.f;
     // where the lattice has a plan for the resident steps they are timed
     // beside the shapes (as shape index n, on the default shape)
     const bool can_stay = !c->plan.tiles.empty() && c->force_model == 0;
     if (can_stay && n < 16) step_default_shape(L, &tx[n], &ty[n]);
     lbm_status st = snapshot(c, snap, true);
+    const bool saved = st == LBM_OK;
     cudaError_t e = cudaSuccess;
     if (st == LBM_OK) e = cudaEventCreate(&e0);
     if (st == LBM_OK && e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -736,35 +739,44 @@ lbm_status lbm_autotune(lbm_ctx *c, int nsteps, int *best_tx, int *best_ty)
         // the shapes of the force model in use, timed with its step
         if (!step_shape_supported(L.precision, tx[k], ty[k])) continue;
         if (c->force_model == 1 && !pt_shape_supported(L.precision, tx[k], ty[k])) continue;
+        const bool stay = k == n;
+        const int timed = stay && nsteps < RESIDENT_TIMED ? RESIDENT_TIMED : nsteps;
         L.tx = tx[k];
         L.ty = ty[k];
         refresh_maps(c);
         st = snapshot(c, snap, false);
         c->t = t0;
-        c->resident = k == n;
-        for (int w = 0; w < 2 && e == cudaSuccess; ++w, ++c->t)
+        c->resident = stay;
+        // outside the timing: two steps, or a resident launch, which takes the
+        // exchange words and loads the kernel; none here: not a candidate
+        if (stay && resident_steps(c, c->plan.min_steps) == 0) continue;
+        for (int w = 0; w < 2 && !stay && e == cudaSuccess; ++w, ++c->t)
             e = launch_one_step(c, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-        int s = resident_steps(c, nsteps);
-        for (; s < nsteps && e == cudaSuccess; ++s, ++c->t)
+        int s = resident_steps(c, timed);
+        if (stay && s == 0) continue;
+        for (; s < timed && e == cudaSuccess; ++s, ++c->t)
             e = launch_one_step(c, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e == cudaSuccess && (best < 0 || ms < best_ms)) {
+        const float us = 1e3f * ms / timed;
+        if (e == cudaSuccess && (best < 0 || us < best_us)) {
             best = k;
-            best_ms = ms;
+            best_us = us;
         }
     }
-    if (st == LBM_OK && e == cudaSuccess && best >= 0) {
-        L.tx = tx[best];
-        L.ty = ty[best];
-        c->resident = best == n;
+    const bool found = st == LBM_OK && e == cudaSuccess && best >= 0;
+    if (saved) {  // the state, on the shape found (on a failure: as it was)
+        L.tx = found ? tx[best] : tx0;
+        L.ty = found ? ty[best] : ty0;
+        c->resident = found && can_stay ? best == n : resident0;
         refresh_maps(c);
-        st = snapshot(c, snap, false);
         c->t = t0;
-        if (st == LBM_OK) e = cudaStreamSynchronize(c->stream);
+        const lbm_status st2 = snapshot(c, snap, false);
+        if (st == LBM_OK) st = st2;
+        if (st == LBM_OK && e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);

@@ -36,6 +36,11 @@ inline int resident_min(int prec, long long nodes)
 {
     return prec == P_F64 || nodes <= 100000 ? 4 : 24;
 }
+// Autotuning times them over this many steps at least, whatever number it is
+// asked for (per step they are compared with the tile kernels): the loading
+// and storing of a call then counts as in the calls of a run, 0.2 to 0.6 us a
+// step, and the least number of steps above is always reached.
+constexpr int RESIDENT_TIMED = 64;
 // A launch takes at most this many, so that no kernel holds the GPU for long.
 constexpr int RESIDENT_MAX = 4096;
 
