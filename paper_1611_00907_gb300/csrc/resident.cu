@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <new>
 
 #include "resident.h"
 
@@ -120,9 +121,9 @@ size_t xchg_bytes(const Lattice &L)
     return 2 * 9 * (size_t)L.plane * 2 * rho_bytes(L.precision);
 }
 
-bool resident_plan(const Lattice *lats, int count, int device, ResidentPlan *p)
+namespace {
+bool make_plan(const Lattice *lats, int count, int device, ResidentPlan *p)
 {
-    *p = ResidentPlan{};
     if (count < 1 || device < 0 || device >= MAX_DEVICES) return false;
     const int prec = lats[0].precision;
     if (prec == P_F16_OFF) return false;
@@ -178,6 +179,20 @@ bool resident_plan(const Lattice *lats, int count, int device, ResidentPlan *p)
     p->device = device;
     p->precision = prec;
     return (int)p->tiles.size() <= sms;
+}
+}  // namespace
+
+// No exception leaves it (its callers are C entries): a host without memory
+// for a plan steps on the tile kernels.
+bool resident_plan(const Lattice *lats, int count, int device, ResidentPlan *p)
+{
+    *p = ResidentPlan{};
+    try {
+        if (make_plan(lats, count, device, p)) return true;
+    } catch (const std::bad_alloc &) {
+    }
+    *p = ResidentPlan{};
+    return false;
 }
 
 cudaError_t launch_resident(const ResidentPlan &p, const Lattice *single, const Lattice *d_lats,
