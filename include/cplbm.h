@@ -144,7 +144,9 @@ lbm_status lbm_set_force_model(lbm_ctx *ctx, int model);
 /* Set the state to equilibrium populations f_i = f_i^eq(rho, u) (Eq. 14)
  * at every fluid node, and the step counter to 0.  rho must be positive and
  * below the EOS's repulsive pole at fluid nodes; ux and uy may be NULL
- * (zero velocity).  Values on solid rows are ignored. */
+ * (zero velocity).  Values on solid rows are ignored.  Steps in FP32
+ * arithmetic take densities below 2^-126 = 1.2e-38 as zero (the lattice
+ * turns non-finite); fields and sums read them back as they are. */
 lbm_status lbm_init(lbm_ctx *ctx, const double *rho, const double *ux,
                     const double *uy, int on_device);
 

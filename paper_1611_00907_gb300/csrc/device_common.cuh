@@ -174,12 +174,15 @@ __device__ __forceinline__ double log_tab(double x)
 
 // Reciprocal, division and logarithm of the arithmetic type: the FP32
 // kernels use the hardware's approximate forms, whose few-ulp errors sit far
-// below the FP32 storage error, with subnormal operands read as zero (a
-// density that small has no finite reciprocal either): one instruction each,
-// where __fdividef and __logf wrap them in the scaling of subnormals, which
-// the issue-bound FP16-storage step paid for (2048 x 1026 walled: 28.1 ->
-// 26.7 us, results unchanged to the bit); FP64 the reciprocal
-// and logarithm above, within one or two ulp of IEEE division and log().
+// below the FP32 storage error.  In the step kernels subnormal operands read
+// as zero: one instruction each, where the scaling of subnormals takes three
+// or four, which the issue-bound FP16-storage step paid for (2048 x 1026
+// walled: 28.1 -> 26.7 us; results of normal operands are the same bits), so
+// a step needs densities of 2^-126 = 1.2e-38 or more (below a quarter of that
+// 1 / rho is infinite in FP32 anyway).  ANY: the logarithm of any density, for
+// the field kernels, which read back whatever a lattice was given.  FP64: the
+// reciprocal and logarithm above, within one or two ulp of IEEE division and
+// log().
 __device__ __forceinline__ float frcp(float x)
 {
     float r;
@@ -189,44 +192,48 @@ __device__ __forceinline__ float frcp(float x)
 __device__ __forceinline__ double frcp(double x) { return rcp_nr(x); }
 __device__ __forceinline__ float fdiv(float a, float b) { return a * frcp(b); }
 __device__ __forceinline__ double fdiv(double a, double b) { return a * rcp_nr(b); }
+template <bool ANY = false>
 __device__ __forceinline__ float flog(float x)
 {
     float l;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x));
+    if constexpr (ANY) asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(x));
+    else asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x));
     return l * 0.693147180559945f;
 }
 __device__ __forceinline__ double flog(double x) { return log_tab(x); }
 
+template <bool ANY = false>
 __device__ __forceinline__ float mu_bulk(const EosT<float> &e, float rho)
 {
     switch (e.kind) {
     case EOS_VDW: {
         const float iq = fdiv(1.0f, 1.0f - e.b * rho);
-        return e.RT * (flog(rho * iq) + iq) - 2.0f * e.a * rho;
+        return e.RT * (flog<ANY>(rho * iq) + iq) - 2.0f * e.a * rho;
     }
     case EOS_CS: {
         const float h = e.quarter_b * rho;
         const float iq = fdiv(1.0f, 1.0f - h);
-        return e.RT * ((3.0f - h) * (iq * iq * iq) + flog(rho) + 1.0f) -
+        return e.RT * ((3.0f - h) * (iq * iq * iq) + flog<ANY>(rho) + 1.0f) -
                2.0f * e.a * rho;
     }
     case EOS_PR: {
         const float br = e.b * rho;
         const float iq = fdiv(1.0f, 1.0f - br);
-        return e.RT * flog(rho * iq) -
+        return e.RT * flog<ANY>(rho * iq) -
                e.pr_c * flog(fdiv(e.pr_s2m1 + br, e.pr_s2p1 - br)) +
                e.RT * iq - fdiv(e.aalpha * rho, 1.0f + 2.0f * br - br * br);
     }
     default: {  // EOS_RKS
         const float br = e.b * rho;
         const float iq = fdiv(1.0f, 1.0f - br);
-        return e.RT * (flog(rho * iq) + iq) - e.rks_c * flog(1.0f + br) -
+        return e.RT * (flog<ANY>(rho * iq) + iq) - e.rks_c * flog(1.0f + br) -
                fdiv(e.aalpha * rho, 1.0f + br);
     }
     }
 }
 
 // FP64: the same with fewer instructions.
+template <bool = false>
 __device__ __forceinline__ double mu_bulk(const EosT<double> &e, double rho)
 {
     switch (e.kind) {
@@ -600,10 +607,12 @@ __device__ __forceinline__ void grad12(const T *s, int c, T &gx, T &gy)
     grad12(row_of(s, c + W), row_of(s, c), row_of(s, c - W), gx, gy);
 }
 // mu = psi'(rho) - kappa lap(rho) (Eq. 8) from the absolute density and 6 lap.
+template <bool ANY = false>
 __device__ __forceinline__ float mu_of(const Consts<float> &K, float rho, float l6)
 {
-    return mu_bulk(K.eos, rho) - K.kappa * (l6 * (1.0f / 6.0f));
+    return mu_bulk<ANY>(K.eos, rho) - K.kappa * (l6 * (1.0f / 6.0f));
 }
+template <bool = false>
 __device__ __forceinline__ double mu_of(const Consts<double> &K, double rho, double l6)
 {
     return K.nk6 * l6 + mu_bulk(K.eos, rho);
@@ -612,7 +621,7 @@ __device__ __forceinline__ double mu_of(const Consts<double> &K, double rho, dou
 // Fill s_mu[(TY + 2) x (TX + 2)] with mu on the tile and a one-node halo
 // (Eq. 8) from the stored-form densities in s_rho; solid rows carry the
 // surface values (Sec. IV, V).
-template <class S, int TX, int TY>
+template <class S, int TX, int TY, bool ANY = false>
 __device__ void mu_tile(const Lattice &L, int X0, int Y0,
                         const typename S::real *s_rho, typename S::real *s_mu)
 {
@@ -635,14 +644,14 @@ __device__ void mu_tile(const Lattice &L, int X0, int Y0,
         } else if (L.walls && r == L.nyf) {
             if (L.top_mode == 0) {
                 const int cb = c - WR;  // fluid neighbour below (row nyf-1)
-                m = mu_of(K, s_rho[cb] + ref, lap6<real, WR>(s_rho, cb));
+                m = mu_of<ANY>(K, s_rho[cb] + ref, lap6<real, WR>(s_rho, cb));
             } else {
                 m = K.mu_top;
             }
         } else if (L.walls && (r < -1 || r > L.nyf)) {
             m = real(0);
         } else {
-            m = mu_of(K, s_rho[c] + ref, lap6<real, WR>(s_rho, c));
+            m = mu_of<ANY>(K, s_rho[c] + ref, lap6<real, WR>(s_rho, c));
         }
         s_mu[k] = m;
     }
