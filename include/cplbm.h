@@ -157,8 +157,13 @@ lbm_status lbm_init(lbm_ctx *ctx, const double *rho, const double *ux,
  * fits the shared memory of all SMs together (FP64 up to about 270 000 nodes,
  * FP32 storage with walls, or once lbm_autotune has found it faster, about
  * 500 000; not FP16, the pressure-tensor force or a chosen tile shape) run as
- * one cooperative launch that keeps the state there; such launches follow one
- * another on a device.  Otherwise blocks of 16 steps replay a CUDA graph
+ * one cooperative launch that keeps the state there.  A periodic lattice in
+ * FP32 storage keeps the tile kernels until autotuned because another order
+ * of sums moves the flow of a phase separation by as much as FP32 is off there
+ * anyway (1e-4 after 340 steps).  On-chip launches of one device follow one
+ * another: lattices on streams of their own overlap only on the tile kernels
+ * (lbm_set_tile), which from four lattices of 256x128 (FP32) or 256x256 (FP64)
+ * on is faster, up to twice; many small lattices belong in a batch.  Otherwise blocks of 16 steps replay a CUDA graph
  * captured on a private stream at the first such call (and again after any
  * change of tile shape, physics, force model or wait limit); while the
  * context's stream is being captured by the caller, every step is a plain
@@ -234,7 +239,8 @@ lbm_status lbm_batch_init(lbm_batch *b, int index, const double *rho,
 /* Queue nsteps steps of every active lattice; all must be initialised.  Four
  * steps or more (24, as for lbm_step) of lattices that together fit the shared memory of all SMs
  * run on the chip, as lbm_step's (not after lbm_batch_set_tile or
- * lbm_batch_schedule with a schedule); the batch takes the memory of the words
+ * lbm_batch_schedule with a schedule), periodic lattices in FP32 storage
+ * included; the batch takes the memory of the words
  * their tiles exchange at the first such call, and steps as other batches do
  * where it is not to be had. */
 lbm_status lbm_batch_step(lbm_batch *b, int nsteps);

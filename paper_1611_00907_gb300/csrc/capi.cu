@@ -487,14 +487,8 @@ lbm_status ctx_create(const lbm_config *cfg, bool alone, lbm_ctx **out)
     alloc((void **)&c->d_prev, (size_t)L.nx * L.ny * sizeof(double));
     const char *no_tma = getenv("CPLBM_NO_TMA");
     c->use_tma = !(no_tma && no_tma[0] == '1');
-    // A periodic FP32 lattice by itself, the set-up of phase separation from a
-    // uniform state, takes the resident steps only when autotuned: that
-    // growth amplifies roundings, and the order of the resident sums left the
-    // velocities of a 387 x 171 lattice 4e-5 from the tile kernels' after 340
-    // steps, though both as far from FP64.
     c->resident = alone && c->use_tma && st == LBM_OK &&
-                  resident_plan(&L, 1, c->device, &c->plan) &&
-                  (L.walls || L.precision == P_F64);
+                  resident_plan(&L, 1, c->device, &c->plan) && resident_alone(L);
     // the densities' row padding is loaded with the tiles and never written:
     // zero, once
     for (int k = 0; k < 2 && st == LBM_OK; ++k)

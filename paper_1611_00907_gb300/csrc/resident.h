@@ -41,6 +41,17 @@ inline int resident_min(int prec, long long nodes)
 // and storing of a call then counts as in the calls of a run, 0.2 to 0.6 us a
 // step, and the least number of steps above is always reached.
 constexpr int RESIDENT_TIMED = 64;
+// Whether a lattice by itself that has a plan takes them without having been
+// autotuned: all but a periodic FP32 one.  That is not for accuracy.  Any other
+// order of sums moves the results of a phase separation from a uniform state,
+// which such a lattice is often set up for and which amplifies every rounding:
+// velocities of 387 x 171 after 342 steps 1.0e-4 (of their norm) from the 64 x
+// 16 tiles', where either is 1.0 to 1.2e-4 from 64 bits.  A Simulation keeps
+// the results it had there until it is autotuned.  A batch takes the resident
+// steps on any lattice: its results there were never a Simulation's (its 32 x
+// 32 tiles are 9e-5 from the 64 x 16 ones too), and the drops, slabs and walls
+// of sweeps move by 1e-6; lbm_batch_set_tile keeps the tile kernels.
+inline bool resident_alone(const Lattice &L) { return L.walls || L.precision == P_F64; }
 // A launch takes at most this many, so that no kernel holds the GPU for long.
 constexpr int RESIDENT_MAX = 4096;
 

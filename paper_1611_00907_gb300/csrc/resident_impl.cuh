@@ -12,7 +12,7 @@
 // that every SM gets one rectangle, of any size, and a step costs the
 // arithmetic of that rectangle plus one trip through L2.  Measured per step,
 // tile kernels (default shape, 16-step graphs) -> here: FP32 64 x 64 20.9 ->
-// 1.7 us, 256 x 128 6.7 -> 2.7, 512 x 512 7.5 -> 5.2, 704 x 704 9.6 -> 8.2;
+// 1.7 us, 256 x 128 6.7 -> 2.5, 512 x 512 7.5 -> 5.2, 704 x 704 9.6 -> 8.2;
 // FP64 64 x 64 47 -> 5.6 us, 256 x 256 39 -> 21, 500 x 200 40 -> 28, 512 x 512
 // 74 -> 64.  What bounds it: up to some 30 000 nodes the exchange and the
 // barriers (about 1.5 us), beyond that FP64 the FP64 units, FP32 issue.
